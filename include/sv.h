@@ -71,8 +71,8 @@ enum {
 /* Options.  Zero-initialised fields take the defaults in brackets. */
 typedef struct {
   int fuse_k;     /* qubits per register group besides qubit 0 (plain) or per fused   */
-                  /* block (tensor cores), 1..5; 0 = the default 5 (plain kernels     */
-                  /* compiled per plan use at most 4).  The tensor-core precisions    */
+                  /* block (tensor cores), 1..5; 0 = the default 5 (the plain kernels  */
+                  /* use at most 4).  The tensor-core precisions    */
                   /* take 5 (32x32 stage unitaries) or 4 (16x16, 12-qubit tiles only);  */
                   /* any other value is SV_ERR_ARG.                                    */
   int precision;  /* SV_PREC_*                                            [PLAIN]       */
@@ -87,8 +87,8 @@ typedef struct {
                   /* sv_apply_batch: the tile size.                                    */
   void *stream;   /* cudaStream_t used by the handle                      [legacy 0]    */
   int tile_bits;  /* qubits per gathered tile, 6..14 (14: plan-specialised kernels    */
-                  /* only) [12 on plan-specialised and tensor-core kernels, 13 on the  */
-                  /* interpreting kernel]                                              */
+                  /* only) [12 on plan-specialised and tensor-core kernels, 11..13 by  */
+                  /* the state's size on the interpreting kernel]                      */
   int low_bits;   /* contiguous low qubits in every tile (coalescing)     [4]           */
   int jit;        /* plain path: run each plan on kernels compiled for it at run time */
                   /* (NVRTC; cached in memory and in the library's directory):       */

@@ -12,7 +12,8 @@ namespace svk {
 // One pass of one circuit.
 struct BatchCP {
   uint64_t state_off;  // float2 offset of the circuit's state in the batch buffer
-  uint32_t pass;       // index into the batch plan's pass array
+  uint32_t block;        // offset of the pass's block (interp_dev.h) in the batch program
+  uint32_t block_bytes;
   uint32_t prev;       // BatchCP index of the circuit's previous pass (kNoPrev if first)
   uint32_t tiles;      // tiles of this pass
   uint32_t circuit;
@@ -30,10 +31,10 @@ struct BatchItem {
 // Device words of one launch: [0] next item, [1] error flag, then one done counter per cp.
 constexpr int kBatchHeader = 2;
 
-// wait_ns: limit of one dependency wait (after which the error word is set and the CTA
+// blocks: the circuit-passes' programs (max_block_bytes: the largest).  wait_ns: limit of one dependency wait (after which the error word is set and the CTA
 // leaves); max_grid > 0 caps the number of CTAs.
-cudaError_t launch_batch(float2 *states, const DevPlanView &plan, const BatchCP *cps, const BatchItem *items,
-                         uint64_t n_items, unsigned int *words, int m, cudaStream_t st,
+cudaError_t launch_batch(float2 *states, const unsigned char *blocks, uint32_t max_block_bytes, const BatchCP *cps,
+                         const BatchItem *items, uint64_t n_items, unsigned int *words, int m, cudaStream_t st,
                          unsigned long long wait_ns = 5000000000ull, int max_grid = 0);
 int batch_block_threads(int m);
 

@@ -9,6 +9,7 @@
 
 #include "../../include/sv.h"
 #include "capi_util.h"
+#include "interp.h"
 #include "jit.h"
 #include "kernels.h"
 #include "plan.h"
@@ -55,9 +56,30 @@ svp::Options plan_options(const sv_options &o) {
   p.pack = !p.fused;  // the plain kernel runs packed plans
   // register qubits per thread of the tile kernels (packed: besides qubit 0; tensor
   // cores: the block size, 5 or 4 qubits)
-  p.rk = p.pack ? svk::tile_pass_register_slots() : (o.fuse_k == 4 ? 4 : 5);
+  p.rk = p.pack ? 4 : (o.fuse_k == 4 ? 4 : 5);
   p.r = std::min(o.fuse_k > 0 ? o.fuse_k : p.rk, p.rk);
   return p;
+}
+
+// Tile size and register slots of a plan on the interpreting kernel where the options leave
+// both open.  Measured on one GB300, us per circuit of depth 16 from |0..0> / 12 on a loaded
+// state, by (register slots, tile qubits):
+//   10 qubits  (2,10) 13.4/13.7  (4,10) 14.8/17.6     one tile: fewer amplitudes a thread
+//              are more warps on the one SM; from 12 qubits the op count weighs more
+//   12         (4,12) 17.8/20.5  (2,12) 21.2/23.2     (2,11) 19.8/24.2
+//   14         (2,11) 22.6/26.7  (4,12) 25.3/28.8     (4,13) 24.6/33.5
+//   16         (4,12) 28.2/30.8  (2,11) 27.3/34.8     (4,13) 31.7/35.5
+//   20         (4,13) 38.8/51.8  (4,12) 45.4/48.3     (128 tiles: one to an SM)
+//   23         (4,12) 164/214    (4,13) 168/212       (4,11) 172/217
+// From 24 qubits (no run-time compiler) passes over HBM weigh most: the largest tile.
+static void interp_shape(const sv_options &o, int n, svp::Options *po) {
+  if (o.tile_bits != 0 || o.fuse_k != 0 || o.low_bits != 0) return;
+  if (n <= 11 || (n >= 13 && n <= 15)) {
+    po->rk = po->r = 2;
+    po->m = 11;
+  } else {
+    po->m = n <= 19 || n == 22 || n == 23 ? 12 : 13;
+  }
 }
 
 svp::Options apply_plan_options(const sv_options &o, int n, bool *want_jit) {
@@ -80,7 +102,7 @@ svp::Options apply_plan_options(const sv_options &o, int n, bool *want_jit) {
   if (po.fused && std::min(po.m, n) < 12) {
     po.fused = false;
     po.pack = true;
-    po.rk = svk::tile_pass_register_slots();
+    po.rk = 4;
     po.r = std::min(po.r, po.rk);
   }
   // plain path: kernels compiled for the plan where they pay (or where asked for), on
@@ -96,6 +118,7 @@ svp::Options apply_plan_options(const sv_options &o, int n, bool *want_jit) {
     const int m = std::min(po.m, n);
     if (o.pipeline >= 0 && po.c == 4 && m >= 10 && m <= 13) po.layout = 1;
   }
+  if (!*want_jit && !po.fused) interp_shape(o, n, &po);
   return po;
 }
 
@@ -277,7 +300,23 @@ sv_status apply_pergate(sv_state *s, const std::vector<svp::Gate> &g) {
 
 namespace svc {
 
-sv_status upload_plan(sv_state *s, const svp::Plan &P, svk::DevPlanView *view) {
+sv_status upload_plan(sv_state *s, const svp::Plan &P, svk::DevPlanView *view, bool interp) {
+  s->block_offset.clear();
+  s->block_bytes.clear();
+  if (interp) {
+    svp::InterpProgram prog;
+    if (!svp::lower_interp(P, &prog)) return fail(SV_ERR_ARG, "the plan has no interpreter form");
+    sv_status st = ensure_device_buffer(&s->d_plan, &s->d_plan_cap, prog.blocks.size());
+    if (st != SV_OK) return st;
+    s->h_plan.assign(prog.blocks.begin(), prog.blocks.end());
+    cudaError_t e = cudaMemcpyAsync(s->d_plan, s->h_plan.data(), s->h_plan.size(), cudaMemcpyHostToDevice, s->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "plan upload");
+    if (s->prof) s->h2d += (double)s->h_plan.size();
+    s->block_offset = prog.offset;
+    s->block_bytes = prog.bytes;
+    *view = svk::DevPlanView{};
+    return SV_OK;
+  }
   auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t o_pass = 0;
   const size_t o_stage = align(o_pass + P.passes.size() * sizeof(svp::DevPass));
@@ -331,7 +370,8 @@ sv_status run_plan(sv_state *s, const svp::Plan &P, const svk::DevPlanView &view
     prof_begin(s);
     cudaError_t e = fused ? svk::launch_fused_pass(s->psi, s->n, view, (int)p, hp, s->stream, f16, P.rk)
                     : jit ? svj::launch_pass(jit, s->psi, s->n, view, (int)p, hp, s->stream, partials, &grid)
-                          : svk::launch_tile_pass(s->psi, s->n, view, (int)p, hp, s->stream);
+                          : svk::launch_tile_pass(s->psi, s->n, static_cast<unsigned char *>(s->d_plan) + s->block_offset[p],
+                                                  s->block_bytes[p], hp.m, P.rk, s->stream);
     prof_end(s, bytes);
     if (jit && s->prof) s->jit_launches += 1;
     if (e != cudaSuccess) { s->broken = true; return cuda_fail(e, "tile pass kernel"); }
@@ -571,7 +611,7 @@ sv_status apply_gates(sv_state *s, const std::vector<svp::Gate> &g) {
       // no compiler: the interpreting kernel, with its register width, on tiles it takes
       po.m = std::min(po.m, svk::tile_pass_max_bits());
       po.layout = 0;
-      po.rk = svk::tile_pass_register_slots();
+      po.rk = 4;
       po.r = std::min(plan_options(s->opts).r, po.rk);
       P = svp::Plan();
       if (!svp::build_plan(s->n, g, po, s->fresh, &P, &err))
@@ -586,7 +626,7 @@ sv_status apply_gates(sv_state *s, const std::vector<svp::Gate> &g) {
     for (const svp::DevPass &dp : P.passes)
       if (dp.stage_count > 256) return fail(SV_ERR_ARG, "fused path: more than 256 stages in one pass");
   svk::DevPlanView view;
-  if ((st = upload_plan(s, P, &view)) != SV_OK) return st;
+  if ((st = upload_plan(s, P, &view, !kfused && !jit)) != SV_OK) return st;
   if ((st = run_plan(s, P, view, kfused, f16, jit)) != SV_OK) return st;
   s->fresh = false;
   if (kfused && (st = check_fused_error(s, view)) != SV_OK) return st;

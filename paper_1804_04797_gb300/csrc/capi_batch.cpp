@@ -20,6 +20,7 @@
 #include "../../include/sv.h"
 #include "batch.h"
 #include "capi_util.h"
+#include "interp.h"
 #include "jit.h"
 #include "kernels.h"
 #include "plan.h"
@@ -128,7 +129,7 @@ struct Batch {
   std::vector<int> nq;
   std::vector<std::unique_ptr<JitCircuit>> jit;
   DeviceBuf states, plan, cps, items, words, chunks, partials, chunk_begin, stats;
-  svk::DevPlanView view{};
+  uint32_t max_block = 0;  // bytes of the largest pass program (plan)
   uint64_t n_items = 0;
   int n_chunks = 0;
   size_t words_bytes = 0;
@@ -288,32 +289,20 @@ sv_status build_batch(const sv_lattice *circs, size_t count, int m_req, int jit,
   po.m = m;
   po.c = 4;
   po.pack = true;  // the batch kernel runs the packed interpreter
-  po.rk = svk::tile_pass_register_slots();
+  po.rk = 4;
   po.r = po.rk;
-  // combined plan
-  std::vector<svp::DevPass> passes;
-  std::vector<svp::DevStage> stages;
-  std::vector<svp::DevOp> ops;
-  std::vector<svp::DevGroupEntry> gtab;
+  // the circuits' pass programs, one after the other
+  svp::InterpProgram prog;
   std::vector<std::vector<uint32_t>> circ_passes(count);
   for (size_t i = 0; i < count; ++i) {
     if (on_jit[i]) continue;
     svp::Plan P;
     const char *err = nullptr;
     if (!svp::build_plan(B->nq[i], gates[i], po, true, &P, &err)) return fail(SV_ERR_ARG, err ? err : "planning failed");
-    const uint32_t sb = (uint32_t)stages.size(), ob = (uint32_t)ops.size();
-    for (svp::DevStage ds : P.stages) {
-      ds.op_begin += ob;  // rebase into the combined arrays
-      stages.push_back(ds);
-    }
-    for (const svp::DevOp &o : P.ops) ops.push_back(o);
-    gtab.insert(gtab.end(), P.gtab.begin(), P.gtab.end());
-    for (svp::DevPass dp : P.passes) {
-      dp.stage_begin += sb;
-      circ_passes[i].push_back((uint32_t)passes.size());
-      passes.push_back(dp);
-    }
+    for (size_t p = 0; p < P.passes.size(); ++p) circ_passes[i].push_back((uint32_t)(prog.offset.size() + p));
+    if (!svp::lower_interp(P, &prog)) return fail(SV_ERR_ARG, "the plan has no interpreter form");
   }
+  for (uint32_t b : prog.bytes) B->max_block = std::max(B->max_block, b);
   // work queue: round r = r-th pass of every circuit that has one, larger circuits first
   std::vector<size_t> order(count);
   for (size_t i = 0; i < count; ++i) order[i] = i;
@@ -328,7 +317,8 @@ sv_status build_batch(const sv_lattice *circs, size_t count, int m_req, int jit,
       if (r >= circ_passes[oi].size()) continue;
       svk::BatchCP cp;
       cp.state_off = state_off[oi];
-      cp.pass = circ_passes[oi][r];
+      cp.block = prog.offset[circ_passes[oi][r]];
+      cp.block_bytes = prog.bytes[circ_passes[oi][r]];
       cp.prev = last_cp[oi];
       cp.tiles = 1u << (B->nq[oi] - m);
       cp.circuit = (uint32_t)oi;
@@ -351,14 +341,8 @@ sv_status build_batch(const sv_lattice *circs, size_t count, int m_req, int jit,
   chunk_begin[count] = (int)chunks.size();
   B->n_chunks = (int)chunks.size();
   // device buffers
-  auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
-  const size_t o_stage = align(passes.size() * sizeof(svp::DevPass));
-  const size_t o_op = o_stage + align(stages.size() * sizeof(svp::DevStage));
-  const size_t o_gt = o_op + align(ops.size() * sizeof(svp::DevOp));
-  const size_t o_err = o_gt + align(gtab.size() * sizeof(svp::DevGroupEntry));
-  const size_t plan_bytes = o_err + 256;
   if ((st = B->states.alloc(total_amps * sizeof(float2))) != SV_OK) return st;
-  if ((st = B->plan.alloc(plan_bytes)) != SV_OK) return st;
+  if ((st = B->plan.alloc(std::max<size_t>(16, prog.blocks.size()))) != SV_OK) return st;
   if ((st = B->cps.alloc(std::max<size_t>(1, cps.size()) * sizeof(svk::BatchCP))) != SV_OK) return st;
   if ((st = B->items.alloc(std::max<size_t>(1, items.size()) * sizeof(svk::BatchItem))) != SV_OK) return st;
   B->words_bytes = (svk::kBatchHeader + cps.size()) * sizeof(unsigned int);
@@ -367,12 +351,8 @@ sv_status build_batch(const sv_lattice *circs, size_t count, int m_req, int jit,
   if ((st = B->partials.alloc(std::max<size_t>(1, chunks.size()) * 2 * sizeof(double))) != SV_OK) return st;
   if ((st = B->chunk_begin.alloc((count + 1) * sizeof(int))) != SV_OK) return st;
   if ((st = B->stats.alloc(std::max<size_t>(1, count) * 2 * sizeof(double))) != SV_OK) return st;
-  std::vector<char> hp(plan_bytes, 0);
-  std::memcpy(hp.data(), passes.data(), passes.size() * sizeof(svp::DevPass));
-  std::memcpy(hp.data() + o_stage, stages.data(), stages.size() * sizeof(svp::DevStage));
-  std::memcpy(hp.data() + o_op, ops.data(), ops.size() * sizeof(svp::DevOp));
-  std::memcpy(hp.data() + o_gt, gtab.data(), gtab.size() * sizeof(svp::DevGroupEntry));
-  cudaError_t e = cudaMemcpy(B->plan.p, hp.data(), plan_bytes, cudaMemcpyHostToDevice);
+  cudaError_t e = cudaSuccess;
+  if (!prog.blocks.empty()) e = cudaMemcpy(B->plan.p, prog.blocks.data(), prog.blocks.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && !cps.empty()) e = cudaMemcpy(B->cps.p, cps.data(), cps.size() * sizeof(svk::BatchCP), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && !items.empty())
     e = cudaMemcpy(B->items.p, items.data(), items.size() * sizeof(svk::BatchItem), cudaMemcpyHostToDevice);
@@ -380,13 +360,6 @@ sv_status build_batch(const sv_lattice *circs, size_t count, int m_req, int jit,
     e = cudaMemcpy(B->chunks.p, chunks.data(), chunks.size() * sizeof(svk::BatchChunk), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(B->chunk_begin.p, chunk_begin.data(), (count + 1) * sizeof(int), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return cuda_fail(e, "sv_apply_batch: upload");
-  char *d = static_cast<char *>(B->plan.p);
-  B->view.passes = reinterpret_cast<const svp::DevPass *>(d);
-  B->view.stages = reinterpret_cast<const svp::DevStage *>(d + o_stage);
-  B->view.ops = reinterpret_cast<const svp::DevOp *>(d + o_op);
-  B->view.mats = reinterpret_cast<const float *>(d + o_err);
-  B->view.err = reinterpret_cast<int *>(d + o_err);
-  B->view.gtab = reinterpret_cast<const svp::DevGroupEntry *>(d + o_gt);
   return SV_OK;
 }
 
@@ -399,7 +372,8 @@ cudaError_t enqueue_batch(Batch *B, cudaStream_t st, bool with_stats) {
   if (e == cudaSuccess && nb) e = cudaEventRecord(B->ev[0], st);
   for (size_t b = 0; e == cudaSuccess && b < nb; ++b) e = cudaStreamWaitEvent(B->branch[b], B->ev[0], 0);
   if (e == cudaSuccess && B->n_items)
-    e = svk::launch_batch(static_cast<float2 *>(B->states.p), B->view, static_cast<const svk::BatchCP *>(B->cps.p),
+    e = svk::launch_batch(static_cast<float2 *>(B->states.p), static_cast<const unsigned char *>(B->plan.p), B->max_block,
+                          static_cast<const svk::BatchCP *>(B->cps.p),
                           static_cast<const svk::BatchItem *>(B->items.p), B->n_items,
                           static_cast<unsigned int *>(B->words.p), B->m, st);
   float2 *states = static_cast<float2 *>(B->states.p);
@@ -568,35 +542,32 @@ extern "C" sv_status sv_selftest_wait_timeout(int limit_ms) {
   if (limit_ms < 1 || limit_ms > 10000) return fail(SV_ERR_ARG, "sv_selftest_wait_timeout: limit_ms must be 1..10000");
   std::lock_guard<std::mutex> lock(g_mu);
   const int m = 13;
-  svp::DevPass dp;
-  std::memset(&dp, 0, sizeof(dp));
-  dp.m = m;
-  dp.c = 4;
-  dp.n = m;
-  for (int i = 0; i < m; ++i) dp.tq[i] = (uint8_t)i;
-  const svk::BatchCP cps[2] = {{0, 0, svk::kNoPrev, 1, 0}, {0, 0, 0, 1, 0}};
+  svp::Options po;
+  po.m = m;
+  po.pack = true;
+  po.rk = po.r = 4;
+  svp::Plan P;
+  svp::InterpProgram prog;
+  const char *err = nullptr;
+  if (!svp::build_plan(m, {}, po, true, &P, &err) || !svp::lower_interp(P, &prog))
+    return fail(SV_ERR_ARG, err ? err : "planning failed");
+  const svk::BatchCP cps[2] = {{0, 0, prog.bytes[0], svk::kNoPrev, 1, 0}, {0, 0, prog.bytes[0], 0, 1, 0}};
   const svk::BatchItem item = {1, 0};  // waits for cp 0, whose tile is never queued
   DeviceBuf state, plan, dcps, ditems, words;
   sv_status st;
   if ((st = state.alloc(sizeof(float2) << m)) != SV_OK) return st;
-  if ((st = plan.alloc(1024)) != SV_OK) return st;
+  if ((st = plan.alloc(prog.blocks.size())) != SV_OK) return st;
   if ((st = dcps.alloc(sizeof(cps))) != SV_OK) return st;
   if ((st = ditems.alloc(sizeof(item))) != SV_OK) return st;
   if ((st = words.alloc((svk::kBatchHeader + 2) * sizeof(unsigned int))) != SV_OK) return st;
-  cudaError_t e = cudaMemcpy(plan.p, &dp, sizeof(dp), cudaMemcpyHostToDevice);
+  cudaError_t e = cudaMemcpy(plan.p, prog.blocks.data(), prog.blocks.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(dcps.p, cps, sizeof(cps), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(ditems.p, &item, sizeof(item), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(words.p, 0, (svk::kBatchHeader + 2) * sizeof(unsigned int));
-  svk::DevPlanView view{};
-  view.passes = static_cast<const svp::DevPass *>(plan.p);
-  view.stages = reinterpret_cast<const svp::DevStage *>(static_cast<char *>(plan.p) + 512);
-  view.ops = nullptr;
-  view.mats = nullptr;
-  view.err = nullptr;
   if (e == cudaSuccess)
-    e = svk::launch_batch(static_cast<float2 *>(state.p), view, static_cast<const svk::BatchCP *>(dcps.p),
-                          static_cast<const svk::BatchItem *>(ditems.p), 1, static_cast<unsigned int *>(words.p), m, 0,
-                          (unsigned long long)limit_ms * 1000000ull, 1);
+    e = svk::launch_batch(static_cast<float2 *>(state.p), static_cast<const unsigned char *>(plan.p), prog.bytes[0],
+                          static_cast<const svk::BatchCP *>(dcps.p), static_cast<const svk::BatchItem *>(ditems.p), 1,
+                          static_cast<unsigned int *>(words.p), m, 0, (unsigned long long)limit_ms * 1000000ull, 1);
   unsigned int hw[svk::kBatchHeader] = {0, 0};
   if (e == cudaSuccess) e = cudaMemcpy(hw, words.p, sizeof(hw), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(e, "sv_selftest_wait_timeout");

@@ -441,7 +441,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
               ";\n";
   std::ostringstream os;
   os << "// pipelined tile-pass kernel of one pass of a plan\n#define SV_PACK_R " << kpr
-     << "\n#define SV_PLAN_KERNELS 1\n#include \"tile_pack.cuh\"\n#include \"tile_pipe.cuh\"\n"
+     << "\n#include \"tile_pack.cuh\"\n#include \"tile_pipe.cuh\"\n"
      << (mma ? "#include \"tile_mma.cuh\"\n" : "")
      << "using namespace svk::tpk;\nusing namespace svk::tpipe;\n" << (mma ? "using namespace svk::tmma;\n" : "");
   if (mma) {
@@ -883,7 +883,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
 std::string pass_source(const svp::Plan &P, int kpr, int pass, bool inner) {
   std::ostringstream os;
   os << "// tile-pass kernel of one pass of a plan\n#define SV_PACK_R " << kpr
-     << "\n#define SV_PLAN_KERNELS 1\n#include \"tile_pack.cuh\"\nusing namespace svk::tpk;\n";
+     << "\n#include \"tile_pack.cuh\"\nusing namespace svk::tpk;\n";
   {
     const size_t pi = (size_t)pass;
     const svp::DevPass &dp = P.passes[pi];

@@ -7,18 +7,19 @@
 // queue holds all circuits' first passes, then all second passes, ..., so the waits are
 // rare and short.  The state is read through L2 only (cp.async.cg), because other CTAs
 // of the same launch wrote it and L1 is not coherent across SMs.  The tile pass is the
-// packed interpreter of the single-circuit path (tile_pack.cuh).
+// interpreter of the single-circuit path (tile_interp.cuh).
 #include <cuda_runtime.h>
 
 #include "batch.h"
 #include "kernels.h"
-#define SV_PACK_R 4
-#include "tile_pack.cuh"
+#include "tile_interp.cuh"
 
 namespace svk {
 namespace {
 
-using namespace tpk;
+using namespace itp;
+
+constexpr int kBatchSlots = 4;  // register slots besides the pack bit
 
 __device__ __forceinline__ unsigned long long now_ns() {
   unsigned long long t;
@@ -33,13 +34,12 @@ __device__ __forceinline__ unsigned int load_acquire(const unsigned int *p) {
 }
 
 __global__ void __launch_bounds__(256, 2)
-batch_kernel(float2 *__restrict__ states, DevPlanView plan, const BatchCP *__restrict__ cps,
-             const BatchItem *__restrict__ items, uint64_t n_items, unsigned int *words,
+batch_kernel(float2 *__restrict__ states, const unsigned char *__restrict__ blocks, const BatchCP *__restrict__ cps,
+             const BatchItem *__restrict__ items, uint64_t n_items, unsigned int *words, uint32_t tile_bytes,
              unsigned long long wait_ns) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4 *tile = reinterpret_cast<float4 *>(smem_raw);
-  __shared__ DevPass P;
-  __shared__ uint64_t chunk_off[1 << 10];
+  unsigned char *blk = smem_raw + tile_bytes;
   __shared__ unsigned int s_item;
   __shared__ int s_stop;
   const int tid = threadIdx.x;
@@ -55,10 +55,9 @@ batch_kernel(float2 *__restrict__ states, DevPlanView plan, const BatchCP *__res
     if (idx >= n_items) break;
     const BatchItem it = items[idx];
     const BatchCP cp = cps[it.cp];
+    const unsigned char *src = blocks + cp.block;
     if (it.cp != cur_cp) {
-      if (tid == 0) P = plan.passes[cp.pass];
-      __syncthreads();
-      build_chunk_table(P, chunk_off);
+      fetch_block(blk, src, cp.block_bytes);
       cur_cp = it.cp;
     }
     if (tid == 0 && cp.prev != kNoPrev) {
@@ -76,13 +75,7 @@ batch_kernel(float2 *__restrict__ states, DevPlanView plan, const BatchCP *__res
     }
     __syncthreads();
     if (s_stop) break;
-    float2 *psi = states + cp.state_off;
-    if (!(P.flags & (svp::PF_INIT_UNIFORM | svp::PF_INIT_ZERO))) {
-      load_tile_async(psi, tile, P, chunk_off, tile_base(P, it.tile));
-      finish_tile_load(tile);
-      __syncthreads();
-    }
-    process_tile(psi, plan, P, chunk_off, tile, it.tile);
+    process_tile<kBatchSlots>(states + cp.state_off, blk, src, tile, it.tile);
     __threadfence();  // each thread's stores visible device-wide before the count
     __syncthreads();
     if (tid == 0) atomicAdd(&done[it.cp], 1u);
@@ -151,28 +144,28 @@ __global__ void batch_stats_final(const double *partials, const int *chunk_begin
 
 }  // namespace
 
-int batch_block_threads(int m) { return 1 << (m - 1 - kPR); }
+int batch_block_threads(int m) { return 1 << (m - 1 - kBatchSlots); }
 
-cudaError_t launch_batch(float2 *states, const DevPlanView &plan, const BatchCP *cps, const BatchItem *items,
-                         uint64_t n_items, unsigned int *words, int m, cudaStream_t st,
+cudaError_t launch_batch(float2 *states, const unsigned char *blocks, uint32_t max_block_bytes, const BatchCP *cps,
+                         const BatchItem *items, uint64_t n_items, unsigned int *words, int m, cudaStream_t st,
                          unsigned long long wait_ns, int max_grid) {
   static bool configured = false;
-  static int per_sm = 1;
-  const size_t smem = sizeof(float2) << 13;  // tiles of <= 13 qubits (capi_batch)
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (!configured) {  // tiles of <= 13 qubits (capi_batch)
+    cudaError_t e = cudaFuncSetAttribute(
+        batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        (int)((sizeof(float2) << 13) + svp::kInterpResident + svp::kInterpPad));
     if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel, 256, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
     configured = true;
   }
+  const size_t tile_bytes = sizeof(float2) << m;
+  const size_t smem = tile_bytes + svp::interp_smem_max(max_block_bytes) + svp::kInterpPad;
   const int threads = batch_block_threads(m);
-  // smaller tiles use fewer threads: more CTAs fit, but the occupancy query for 256
-  // threads is a safe lower bound
-  int grid = device_sm_count() * per_sm * (256 / threads);
+  int per_sm = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel, threads, smem);
+  if (e != cudaSuccess) return e;
+  int grid = device_sm_count() * (per_sm < 1 ? 1 : per_sm);
   if (max_grid > 0 && grid > max_grid) grid = max_grid;
-  batch_kernel<<<grid, threads, sizeof(float2) << m, st>>>(states, plan, cps, items, n_items, words, wait_ns);
+  batch_kernel<<<grid, threads, smem, st>>>(states, blocks, cps, items, n_items, words, (uint32_t)tile_bytes, wait_ns);
   return cudaGetLastError();
 }
 

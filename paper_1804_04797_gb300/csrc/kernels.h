@@ -17,12 +17,11 @@ struct Mat2 {
 // K0: write |0..0> (uniform == false) or the uniform 2^{-n/2} state.  Write-only.
 cudaError_t launch_init(float2 *psi, int n, bool uniform, float amp, cudaStream_t st);
 
-// K1/K2/K3 plain tile pass: one sweep over all tiles of one pass of a packed plan.
-// host_pass is the host copy of the same pass (tile shape, flags).
-cudaError_t launch_tile_pass(float2 *psi, int n, const DevPlanView &plan, int pass_index,
-                             const svp::DevPass &host_pass, cudaStream_t st);
-// Register slots besides the pack bit of the packed plain kernel (the planner's rk).
-int tile_pass_register_slots();
+// K1/K2/K3 plain tile pass, interpreted: one sweep over all tiles (m qubits) of one pass;
+// block: the pass's program in device memory (interp_dev.h), of `bytes` bytes; rk: the
+// plan's register slots (2..4).
+cudaError_t launch_tile_pass(float2 *psi, int n, const unsigned char *block, uint32_t bytes, int m, int rk,
+                             cudaStream_t st);
 // Largest tile (qubits) of the interpreting plain kernel; the plan-specialised kernels
 // take up to svp::kMaxTileBits.
 int tile_pass_max_bits();

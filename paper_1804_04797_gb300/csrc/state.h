@@ -51,6 +51,8 @@ struct sv_state {
   svp::Options plan_po;
   const svj::Module *plan_jit = nullptr;
   svk::DevPlanView plan_view{};
+  // a plan on the interpreting kernel: where each pass's block lies in d_plan
+  std::vector<uint32_t> block_offset, block_bytes;
   // the norm sums (sum p, sum p^2) of the current state, computed by the last pass of a
   // plan-kernel run as it wrote the state: d_sums[0..1]; d_sums[2..] per-CTA partials.
   // Any other write of the state clears sums_valid; a state the caller can write
@@ -79,7 +81,9 @@ svp::Options plan_options(const sv_options &o);
 svp::Options apply_plan_options(const sv_options &o, int n, bool *want_jit);
 sv_status check_options(const sv_options &o);
 sv_status convert_gates(int n, const sv_gate *g, size_t count, bool inverse, std::vector<svp::Gate> *out);
-sv_status upload_plan(sv_state *s, const svp::Plan &P, svk::DevPlanView *view);
+// The plan's device copy (in s->d_plan): as the plan kernels read it, or (interp) as the
+// interpreting kernel does.
+sv_status upload_plan(sv_state *s, const svp::Plan &P, svk::DevPlanView *view, bool interp = false);
 sv_status run_plan(sv_state *s, const svp::Plan &P, const svk::DevPlanView &view, bool fused, bool f16 = false,
                    const svj::Module *jit = nullptr);
 // Apply g to s on plan-specialised kernels whose last pass, instead of storing the state,

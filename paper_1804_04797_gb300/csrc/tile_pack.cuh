@@ -1,4 +1,5 @@
-// Packed plain tile pass: the register form of the fp32 CUDA-core kernel.
+// Packed plain tile pass: the register form of the fp32 CUDA-core kernels compiled for a
+// plan (the interpreting kernels' is in tile_interp.cuh).
 //
 // A thread holds 32 PAIRS of amplitudes.  The two amplitudes of a pair differ only in
 // tile bit 0 (the pack bit, always qubit 0: two neighbours in memory), and a pair is
@@ -427,161 +428,14 @@ __device__ __forceinline__ void phase_all(Regs &R, Regs &I, int p) {
   }
 }
 
-#ifndef SV_PLAN_KERNELS  // the interpreter: not needed by the kernels compiled for one plan
-// One op by its flat code.  `cond`: the op's condition on the thread's fixed qubits.
-// Signs and projectors of conditional diagonal ops become factors (1 where the
-// condition fails); scalar phases and zeroing of the group are only recorded.  The
-// planner makes every other kind of op unconditional in a packed plan and emits no
-// general 2x2 op for the gate set.
-#define SV_P6(M, A) M(A, 0) M(A, 1) M(A, 2) M(A, 3) M(A, 4)
-#define SV_PAIR_CASE(G, J) case svp::P_PAIR + 6 * G##_I + J: pairs<G, J>(R, I); break;
-#define SV_DIAG_CASE(D, J) case svp::P_DIAG + 6 * D##_I + J: diag<D, J>(R, I, tc); break;
-#define SV_Z_CASE(X, J) \
-  case svp::P_DIAG + 12 + J: factor<J, 1>(R, I, fz); break; \
-  case svp::P_DIAG + 18 + J: factor<J, 1>(R, I, f0); break; \
-  case svp::P_DIAG + 24 + J: factor<J, 0>(R, I, f0); break;
-#define SV_TWO_CASE(J, K) \
-  case svp::P_CZ + 6 * J + K: two<J, K, false>(R, I); break; \
-  case svp::P_PEQ + 6 * J + K: two<J, K, true>(R, I); break;
-
-constexpr int GH_I = 0, GSX_I = 1, GSY_I = 2, GSXDG_I = 3, GSYDG_I = 4, DT1_I = 0, DTDG1_I = 1;
-
-// The op's code and argument (the first word of its 16-byte head).
-__device__ __forceinline__ void apply_op(Regs &R, Regs &I, uint32_t code, uint32_t arg, bool cond, int &ph,
-                                         bool &zero) {
-  using namespace svp;
-  const float fz = cond ? -1.f : 1.f, f0 = cond ? 0.f : 1.f;
-  const float tc = arg ? kS2up : kS2dn;  // T ops: the plan's rounding choice
-  switch (code) {
-    SV_P6(SV_PAIR_CASE, GH)
-    case P_PAIR + 0 + kPackSlot: pairs_pack<GH>(R, I); break;
-    SV_P6(SV_PAIR_CASE, GSX)
-    case P_PAIR + 6 + kPackSlot: pairs_pack<GSX>(R, I); break;
-    SV_P6(SV_PAIR_CASE, GSY)
-    case P_PAIR + 12 + kPackSlot: pairs_pack<GSY>(R, I); break;
-    SV_P6(SV_PAIR_CASE, GSXDG)
-    case P_PAIR + 18 + kPackSlot: pairs_pack<GSXDG>(R, I); break;
-    SV_P6(SV_PAIR_CASE, GSYDG)
-    case P_PAIR + 24 + kPackSlot: pairs_pack<GSYDG>(R, I); break;
-    SV_P6(SV_DIAG_CASE, DT1)
-    case P_DIAG + 0 + kPackSlot: diag_pack<DT1>(R, I, tc); break;
-    SV_P6(SV_DIAG_CASE, DTDG1)
-    case P_DIAG + 6 + kPackSlot: diag_pack<DTDG1>(R, I, tc); break;
-    SV_P6(SV_Z_CASE, 0)
-    case P_DIAG + 12 + kPackSlot: factor_pack<1>(R, I, fz); break;
-    case P_DIAG + 18 + kPackSlot: factor_pack<1>(R, I, f0); break;
-    case P_DIAG + 24 + kPackSlot: factor_pack<0>(R, I, f0); break;
-    SV_TWO_CASE(0, 1) SV_TWO_CASE(0, 2) SV_TWO_CASE(0, 3) SV_TWO_CASE(0, 4) SV_TWO_CASE(0, 5)
-    SV_TWO_CASE(1, 2) SV_TWO_CASE(1, 3) SV_TWO_CASE(1, 4) SV_TWO_CASE(1, 5)
-    SV_TWO_CASE(2, 3) SV_TWO_CASE(2, 4) SV_TWO_CASE(2, 5)
-    SV_TWO_CASE(3, 4) SV_TWO_CASE(3, 5)
-    SV_TWO_CASE(4, 5)
-    case P_PHASE: ph += cond ? (int)arg : 0; break;
-    case P_ZERO: zero = zero || cond; break;
-    case P_SCALE: scale_all(R, I, __int_as_float((127 - (int)arg) << 23)); break;  // 2^-arg, exact
-    case P_GLOBAL:
-      switch (arg & 15u) {
-        case 1: global_factor<1, 0>(R, I); break;
-        case 2: global_factor<2, 0>(R, I); break;
-        case 3: global_factor<3, 0>(R, I); break;
-        case 4: global_factor<4, 0>(R, I); break;
-        case 5: global_factor<5, 0>(R, I); break;
-        case 6: global_factor<6, 0>(R, I); break;
-        case 7: global_factor<7, 0>(R, I); break;
-        case 8: global_factor<0, 1>(R, I); break;
-        case 9: global_factor<1, 1>(R, I); break;
-        case 10: global_factor<2, 1>(R, I); break;
-        case 11: global_factor<3, 1>(R, I); break;
-        case 12: global_factor<4, 1>(R, I); break;
-        case 13: global_factor<5, 1>(R, I); break;
-        case 14: global_factor<6, 1>(R, I); break;
-        case 15: global_factor<7, 1>(R, I); break;
-        default: break;
-      }
-      break;
-    default: break;
-  }
-}
-#undef SV_P6
-#undef SV_PAIR_CASE
-#undef SV_DIAG_CASE
-#undef SV_Z_CASE
-#undef SV_TWO_CASE
-
-// The stage's ops in order; the op after the current one is loaded while it runs (the
-// plan ends with a no-op, so the load after a stage's last op stays inside it).  W: the
-// thread's condition word.
-__device__ __forceinline__ void apply_ops(Regs &R, Regs &I, const DevOp *ops, const DevStage &st, uint32_t W) {
-  int ph = 0;
-  bool zero = false;
-  const uint4 *head = reinterpret_cast<const uint4 *>(ops + st.op_begin);
-  const int stride = sizeof(DevOp) / sizeof(uint4);
-  uint4 h = head[0];
-  for (int o = 0; o < st.op_count; ++o) {
-    const uint4 nxt = head[(o + 1) * stride];
-    apply_op(R, I, h.x & 0xffu, (h.x >> 8) & 0xffu, (W & h.z) == h.w, ph, zero);
-    h = nxt;
-  }
-  if (zero) {
-    scale_all(R, I, 0.f);
-  } else {
-    if (st.halves) scale_all(R, I, __int_as_float((127 - st.halves) << 23));  // 2^-halves, exact
-    if (ph & 7) phase_all(R, I, ph & 7);
-  }
-}
-
-#endif  // SV_PLAN_KERNELS
-
 // ---- addressing ---------------------------------------------------------------------------
 // 16-byte slot of pair k (tile bits 1..m-1): pair bit i toggles slot bit i mod 3, so the
 // 8 lanes of a quarter warp hit distinct 16-byte bank groups when the planner gives them
 // three pair bits of distinct residues.  Linear over XOR.
 __device__ __forceinline__ uint32_t pack_phys(uint32_t k) { return k ^ (((k >> 3) ^ (k >> 6) ^ (k >> 9)) & 7u); }
 
-// Byte offset of group g's first pair.
-__device__ __forceinline__ uint32_t group_base(const DevPlanView &plan, uint32_t si, int g) {
-  const svp::DevGroupEntry *t = plan.gtab + svp::kGroupEntries * si;
-  return t[g & 15].L ^ t[16 + ((g >> 4) & 15)].L ^ t[32 + ((g >> 8) & 15)].L;
-}
-
-__device__ __forceinline__ void load_group(const float4 *tile, const DevPlanView &plan, uint32_t si, uint32_t a0,
-                                           Regs &R, Regs &I) {
-  const svp::DevGroupEntry *t = plan.gtab + svp::kGroupEntries * si + svp::kRegEntry;
-  uint32_t rx[kPR];
-#pragma unroll
-  for (int j = 0; j < kPR; ++j) rx[j] = t[j].L;
-  const char *tb = reinterpret_cast<const char *>(tile);
-#pragma unroll
-  for (int p = 0; p < kP; ++p) {
-    uint32_t a = a0;
-#pragma unroll
-    for (int j = 0; j < kPR; ++j)
-      if ((p >> j) & 1) a ^= rx[j];
-    const float4 x = *reinterpret_cast<const float4 *>(tb + a);
-    R[p] = f2(x.x, x.y);
-    I[p] = f2(x.z, x.w);
-  }
-}
-
-__device__ __forceinline__ void store_group(float4 *tile, const DevPlanView &plan, uint32_t si, uint32_t a0,
-                                            const Regs &R, const Regs &I) {
-  const svp::DevGroupEntry *t = plan.gtab + svp::kGroupEntries * si + svp::kRegEntry;
-  uint32_t rx[kPR];
-#pragma unroll
-  for (int j = 0; j < kPR; ++j) rx[j] = t[j].L;
-  char *tb = reinterpret_cast<char *>(tile);
-#pragma unroll
-  for (int p = 0; p < kP; ++p) {
-    uint32_t a = a0;
-#pragma unroll
-    for (int j = 0; j < kPR; ++j)
-      if ((p >> j) & 1) a ^= rx[j];
-    *reinterpret_cast<float4 *>(tb + a) = make_float4(R[p].x, R[p].y, I[p].x, I[p].y);
-  }
-}
-
-// The same with the register-slot masks given (the kernels compiled for one plan pass
-// them as constants).
+// A group's pairs from / to the tile: a0 the byte offset of its first pair, rx the byte-offset
+// masks of the register slots (constants in the kernels compiled for one plan).
 // kCopied: the tile is still as the asynchronous copies left it, pairs as
 // (re, im, re', im') (the first stage of a pass that read its tile; see finish_tile_load).
 template <bool kCopied = false>
@@ -790,55 +644,6 @@ __device__ __forceinline__ void store_tile(float2 *__restrict__ psi, const float
 __device__ __forceinline__ void init_tile(float4 *tile, const DevPass &P, uint64_t base) {
   init_tile(tile, P, base, threadIdx.x, blockDim.x);
 }
-
-#ifndef SV_PLAN_KERNELS  // the interpreter
-// One tile of one packed pass whose data is in `tile` (or is generated): every stage in
-// registers, then the store.  Ends with __syncthreads.
-__device__ __forceinline__ void process_tile(float2 *__restrict__ psi, const DevPlanView &plan, const DevPass &P,
-                                             const uint64_t *chunk_off, float4 *tile, uint64_t tile_id) {
-  const int tid = threadIdx.x;
-  const uint64_t base = tile_base(P, tile_id);
-  const bool init = (P.flags & (svp::PF_INIT_UNIFORM | svp::PF_INIT_ZERO)) != 0;
-  if (init && P.stage_count == 0) {
-    init_tile(tile, P, base);
-    __syncthreads();
-  }
-  // condition word: the group index below the tile index (n - 1 - kPR <= 32 bits)
-  const uint32_t W = ((uint32_t)tile_id << (P.m - 1 - kPR)) | (uint32_t)tid;
-  for (int s = 0; s < P.stage_count; ++s) {
-    const uint32_t si = P.stage_begin + s;
-    const DevStage &st = plan.stages[si];
-    Regs R, I;
-    if (s == 0 && init) init_regs(R, I, P, W);
-    else load_group(tile, plan, si, group_base(plan, si, tid), R, I);
-    apply_ops(R, I, plan.ops, st, W);
-    // Recompute the address rather than keeping it live across the ops.
-    asm volatile("" ::: "memory");
-    store_group(tile, plan, si, group_base(plan, si, tid), R, I);
-    __syncthreads();
-  }
-  store_tile(psi, tile, P, chunk_off, base);
-  __syncthreads();
-}
-
-// A CTA's sweep over its tiles (tile_id = first, first + stride, ...): read, process.
-// (A second buffer with the next tile's read in flight measured slower: it halves the
-// resident CTAs, and this kernel is bound by latency, not by bandwidth.)
-__device__ __forceinline__ void sweep_tiles(float2 *__restrict__ psi, const DevPlanView &plan, const DevPass &P,
-                                            const uint64_t *chunk_off, float4 *tile, uint64_t first, uint64_t stride,
-                                            uint64_t num_tiles) {
-  const bool init = (P.flags & (svp::PF_INIT_UNIFORM | svp::PF_INIT_ZERO)) != 0;
-  for (uint64_t tile_id = first; tile_id < num_tiles; tile_id += stride) {
-    if (!init) {
-      load_tile_async(psi, tile, P, chunk_off, tile_base(P, tile_id));
-      finish_tile_load(tile);
-      __syncthreads();
-    }
-    process_tile(psi, plan, P, chunk_off, tile, tile_id);
-  }
-}
-
-#endif  // SV_PLAN_KERNELS
 
 }  // namespace tpk
 }  // namespace svk
