@@ -249,9 +249,10 @@ sv_status sv_branch_amplitudes(const sv_lattice *lat, const sv_cut *cut, const u
  * halves' batched branch states A (n_A + t qubits) and B (n_B + t) give
  * psi[x_A + (x_B << n_A)] = sum_l A_l[x_A] B_l[x_B], a complex matrix product over the
  * 2^t branches, written into out (an n-qubit handle on the same device; fp32
- * accumulation).  Crossing CZs that only sign the output are applied to the result as
- * CZ gates; the others are fully decomposed (an implicit decomposition fixes a branch by
- * an output bit, which a product over all outputs cannot).  Half A must be qubits
+ * accumulation).  Unless cut->full_decomposition: the product applies the signs of crossing
+ * CZs that only sign the output, and an implicit decomposition (see sv_branch_amplitudes)
+ * fixes its branch by an output bit for a whole tile of the product, so only the others are
+ * summed over (at least 7 bits of either half stay free of them).  Half A must be qubits
  * 0..n_A-1 (a cut between lattice rows).  SV_ERR_ARG otherwise. */
 sv_status sv_branch_full_state(const sv_lattice *lat, const sv_cut *cut, const sv_options *opts, sv_state *out);
 

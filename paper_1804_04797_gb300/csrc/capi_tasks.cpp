@@ -56,9 +56,9 @@ struct CutPlan {
   std::vector<std::pair<int, int>> fix_b;
 };
 
-// allow_implicit: may a crossing CZ be decomposed implicitly (an amplitude sum can fix
-// the branch index by the output bit; a full-state product cannot)
-sv_status plan_cut(const sv_lattice *lat, const sv_cut *cut, CutPlan *C, bool allow_implicit = true) {
+// full_state: the cut is for the product over all outputs, whose tiles agree in the output bits
+// that fix branches: at least 7 bits of either half are left to a tile's rows and columns.
+sv_status plan_cut(const sv_lattice *lat, const sv_cut *cut, CutPlan *C, bool full_state = false) {
   std::vector<sv_gate> g;
   sv_status st = generate(lat, &g);
   if (st != SV_OK) return st;
@@ -81,13 +81,26 @@ sv_status plan_cut(const sv_lattice *lat, const sv_cut *cut, CutPlan *C, bool al
   // roles: 0 = full (projector on A, Z on B), 1 = absorbed sign, 2 = implicit on A (A's
   // qubit stays a basis state: no branch bit in A), 3 = implicit on B
   std::vector<int> role;
+  uint64_t by_a = 0, by_b = 0;  // the qubits of implicit decompositions
+  const int most_a = full_state ? na - 7 : na, most_b = full_state ? nb - 7 : nb;
   for (size_t i = 0; i < g.size(); ++i) {
     const sv_gate &x = g[i];
     if (x.kind != SV_CZ || C->in_a[x.q0] == C->in_a[x.q1] || x.layer > depth) continue;
     const int qa = C->in_a[x.q0] ? x.q0 : x.q1, qb = C->in_a[x.q0] ? x.q1 : x.q0;
     const bool qa_quiet = last_nd[qa] < (long)i, qb_quiet = last_nd[qb] < (long)i;
     int r = 0;
-    if (!cut->full_decomposition) r = (qa_quiet && qb_quiet) ? 1 : !allow_implicit ? 0 : qa_quiet ? 2 : qb_quiet ? 3 : 0;
+    if (!cut->full_decomposition) {
+      const uint64_t a = by_a | (1ull << qa), b = by_b | (1ull << qb);
+      if (qa_quiet && qb_quiet) {
+        r = 1;
+      } else if (qa_quiet && __builtin_popcountll(a) <= most_a) {
+        r = 2;
+        by_a = a;
+      } else if (qb_quiet && __builtin_popcountll(b) <= most_b) {
+        r = 3;
+        by_b = b;
+      }
+    }
     role.push_back(r);
   }
   C->t = (int)role.size();
@@ -101,7 +114,9 @@ sv_status plan_cut(const sv_lattice *lat, const sv_cut *cut, CutPlan *C, bool al
   C->tf = n_full;
   C->ta = n_full + n_impl_b;  // A carries the Z^l side of CZs implicit on B
   C->tb = n_full + n_impl_a;
-  if (na + C->ta > 34 || nb + C->tb > 34)
+  // (a full state's halves are held to the branch bits of all expanded CZs)
+  const int expanded = full_state ? C->t - C->absorbed : 0;
+  if (na + std::max(C->ta, expanded) > 34 || nb + std::max(C->tb, expanded) > 34)
     return fail(SV_ERR_ARG, "sv_branch_amplitudes: half qubits + branch bits must be <= 34");
   // Half gate lists: every qubit, branch bits included, starts with H, so each branch
   // slice holds its half's state times 2^{-t_half/2}.  Branch bit numbering: the full
@@ -376,7 +391,7 @@ extern "C" sv_status sv_branch_full_state(const sv_lattice *lat, const sv_cut *c
   clear_error();
   if (!lat || !cut || !out) return fail(SV_ERR_ARG, "sv_branch_full_state: NULL argument");
   CutPlan C;
-  sv_status st = plan_cut(lat, cut, &C, false);
+  sv_status st = plan_cut(lat, cut, &C, true);
   if (st != SV_OK) return st;
   if (out->n != C.n) return fail(SV_ERR_ARG, "sv_branch_full_state: output state has the wrong size");
   if (cut->half_a_mask != (C.na >= 64 ? ~0ull : (1ull << C.na) - 1))
@@ -393,29 +408,65 @@ extern "C" sv_status sv_branch_full_state(const sv_lattice *lat, const sv_cut *c
   if ((st = set_device(out)) != SV_OK) return st;
   cudaError_t e = cudaStreamSynchronize(A.s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(B.s->stream);
-  // each branch slice carries 2^{-t/2} per half
-  const float scale = std::ldexp(1.0f, C.tf);
+  // each branch slice of a half carries 2^{-t_half/2} (an odd total leaves a factor sqrt2: hi
+  // and lo parts)
+  const double exact = std::pow(2.0, 0.5 * (C.ta + C.tb));
+  const float2 scale = make_float2((float)exact, (C.ta + C.tb) % 2 ? (float)(exact - (double)(float)exact) : 0.f);
+  svk::OuterShape S;
+  S.nA = C.na;
+  S.nB = C.nb;
+  S.t = C.tf;
+  uint64_t by_a = 0, by_b = 0;  // bits of x_A, x_B that fix branches of the other half
+  for (const auto &f : C.fix_b) {
+    S.fix_b_by[S.fix_b++] = (uint8_t)C.local[f.second];
+    by_a |= 1ull << C.local[f.second];
+  }
+  for (const auto &f : C.fix_a) {
+    S.fix_a_by[S.fix_a++] = (uint8_t)C.local[f.second];
+    by_b |= 1ull << C.local[f.second];
+  }
+  for (int pass = 0, ia = 0, ib = 0; pass < 2; ++pass) {
+    for (int q = 0; q < C.na; ++q)
+      if ((int)((by_a >> q) & 1) == pass) S.a_bit[ia++] = (uint8_t)q;
+    for (int q = 0; q < C.nb; ++q)
+      if ((int)((by_b >> q) & 1) == pass) S.b_bit[ib++] = (uint8_t)q;
+    if (pass == 0) {
+      S.a_free = ia;
+      S.b_free = ib;
+    }
+  }
+  // the crossing CZs taken as output signs ride on the product (they commute with part C:
+  // neither qubit meets a non-diagonal gate after them; an even number on one bond is none,
+  // and at most 33 bonds of a lattice of 64 sites cross a cut between its first n_A qubits
+  // and the rest)
+  std::vector<std::pair<int, int>> odd(C.signs);
+  std::sort(odd.begin(), odd.end());
+  for (size_t i = 0; i < odd.size(); ++i) {
+    if (i + 1 < odd.size() && odd[i] == odd[i + 1]) { ++i; continue; }
+    S.sign_a[S.signs] = (uint8_t)odd[i].first;
+    S.sign_b[S.signs++] = (uint8_t)(odd[i].second - C.na);
+  }
   // the tensor-core precisions: the product on tcgen05 (TF32x3), else on the CUDA cores
   const bool tc = (o.precision == SV_PREC_TF32X3 || o.precision == SV_PREC_F16X3) &&
-                  svk::fused_supported() && svk::outer_sum_tc_supported(C.na, C.nb, C.tf);
+                  svk::fused_supported() && svk::outer_sum_tc_supported(S);
   void *scratch = nullptr;
   int *d_err = nullptr;
   if (e == cudaSuccess && tc) {
-    e = cudaMalloc(&scratch, svk::outer_sum_tc_scratch(C.na, C.nb, C.tf) + 256);
+    e = cudaMalloc(&scratch, svk::outer_sum_tc_scratch(S) + 256);
     if (e == cudaSuccess) {
-      d_err = reinterpret_cast<int *>(static_cast<char *>(scratch) + svk::outer_sum_tc_scratch(C.na, C.nb, C.tf));
+      d_err = reinterpret_cast<int *>(static_cast<char *>(scratch) + svk::outer_sum_tc_scratch(S));
       e = cudaMemsetAsync(d_err, 0, sizeof(int), out->stream);
     } else {
       scratch = nullptr;
     }
     if (e == cudaSuccess) {
       profile_begin(out);
-      e = svk::launch_outer_sum_tc(A.s->psi, C.na, B.s->psi, C.nb, C.tf, scale, out->psi, scratch, d_err, out->stream);
+      e = svk::launch_outer_sum_tc(A.s->psi, B.s->psi, S, scale, out->psi, scratch, d_err, out->stream);
       profile_end(out, std::ldexp(8.0, C.n));
     }
   } else if (e == cudaSuccess) {
     profile_begin(out);
-    e = svk::launch_outer_sum(A.s->psi, C.na, B.s->psi, C.nb, C.tf, scale, out->psi, out->stream);
+    e = svk::launch_outer_sum(A.s->psi, B.s->psi, S, scale, out->psi, out->stream);
     profile_end(out, std::ldexp(8.0, C.n));
   }
   int h_err = 0;
@@ -429,11 +480,6 @@ extern "C" sv_status sv_branch_full_state(const sv_lattice *lat, const sv_cut *c
   if (h_err) { out->broken = true; return fail(SV_ERR_TIMEOUT, "sv_branch_full_state: a tensor-core wait gave up"); }
   out->fresh = false;
   if (out->prof) out->other_launches += 1;
-  // the crossing CZs taken as output signs act on the product state like any CZ
-  // (they commute with part C: neither qubit meets a non-diagonal gate after them)
-  std::vector<svp::Gate> signs;
-  for (const auto &sg : C.signs) signs.push_back(svp::Gate{svp::K_CZ, (uint8_t)sg.first, (uint8_t)sg.second});
-  if (!signs.empty() && (st = apply_gates(out, signs)) != SV_OK) return st;
   // part C (Eq. 3): the layers after the cut depth on the reconstructed state
   if (!C.part_c.empty() && (st = apply_gates(out, C.part_c)) != SV_OK) return st;
   e = cudaStreamSynchronize(out->stream);

@@ -1,7 +1,9 @@
 // The tensor form of the cut decomposition on the tcgen05 tensor cores (Eqs. 6-7):
 //     psi_AB[x_A + 2^nA x_B] = scale * sum_l A_l[x_A] B_l[x_B],
 // i.e. the complex product Psi = Bm Am^T of the half-states' branch matrices Bm (2^nB x L)
-// and Am (2^nA x L), L = 2^t summed branches, as one real GEMM with K = 2L:
+// and Am (2^nA x L), L = 2^t summed branches, as one real GEMM with K = 2L (where a branch is
+// fixed by an output bit, one for every combination of slices, the rows and columns taken
+// in OuterShape's order):
 //     D[x_B, 2 x_A + o] = sum_{l, c} Aop[x_B, 2l + c] Bop[2 x_A + o, 2l + c],
 //     Aop[x_B, 2l + c] = (Re, Im)_c B_l[x_B],
 //     Bop[2 x_A, 2l + c] = (Re A_l[x_A], -Im A_l[x_A])_c,  Bop[2 x_A + 1, 2l + c] = (Im, Re)_c,
@@ -10,8 +12,8 @@
 // Alo Bhi is accumulated in fp32 in tensor memory (the lo*lo term is ~2^-22 relative).
 //
 // A prep kernel writes the split operands as images in the MMA's shared-memory layout
-// (K-major, no swizzle: 8-row x 16-byte core matrices), one contiguous block per (row tile,
-// 32-wide K chunk), so a CTA fetches each with one bulk copy.  The GEMM kernel is
+// (K-major, no swizzle: 8-row x 16-byte core matrices), one contiguous block per (slice, row
+// tile, 32-wide K chunk), so a CTA fetches each with one bulk copy.  The GEMM kernel is
 // persistent (two CTAs per SM: one stores its tile while the other computes): per output
 // tile of 128 x 128 amplitudes it loads the blocks of every K chunk, one thread issues the
 // 3 x 4 MMAs (M = 128, N = 256, K = 8) per chunk, and the warps move D from tensor memory
@@ -48,33 +50,42 @@ __device__ __forceinline__ float tf32_rn(float x) {
   return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
 }
 
-// Operand images.  Aop: row tile rt, chunk kc at ((rt * kch + kc) * 2 + part) * kABlock;
-// Bop likewise with kBBlock.  One thread per (row, k) of each operand.
-__global__ void outer_prep_kernel(const float2 *__restrict__ A, int nA, const float2 *__restrict__ B, int nB, int t,
+// Index bits of x spread over a half's qubits in OuterShape's order.
+__device__ __forceinline__ uint64_t spread(uint64_t i, const uint8_t *bit, int n) {
+  uint64_t x = 0;
+  for (int k = 0; k < n; ++k) x |= ((i >> k) & 1ull) << bit[k];
+  return x;
+}
+
+// Operand images.  Aop: slice s of B, row tile rt, chunk kc at (((s * rtiles + rt) * kch + kc) *
+// 2 + part) * kABlock; Bop likewise with A, its column tiles and kBBlock.  One thread per
+// (slice, row, k) of each operand.
+__global__ void outer_prep_kernel(const float2 *__restrict__ A, const float2 *__restrict__ B, const OuterShape S,
                                   int kch, unsigned char *__restrict__ aimg, unsigned char *__restrict__ bimg) {
-  const uint64_t L = 1ull << t, K = (uint64_t)kch * kKc;
-  const uint64_t na = 1ull << nA, nb = 1ull << nB;
-  const uint64_t nA_ops = nb * K, nB_ops = 2 * na * K;
+  const uint64_t L = 1ull << S.t, K = (uint64_t)kch * kKc;
+  const uint64_t na = 1ull << S.nA, nb = 1ull << S.nB;
+  const uint64_t nA_ops = (nb << S.fix_b) * K, nB_ops = 2 * (na << S.fix_a) * K;
   for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nA_ops + nB_ops;
        e += (uint64_t)gridDim.x * blockDim.x) {
     float v;
     unsigned char *dst;
     uint32_t blk;
-    if (e < nA_ops) {  // Aop[x_B, k]
-      const uint64_t xb = e / K, k = e % K, l = k >> 1;
-      const float2 z = l < L ? B[xb + (l << nB)] : make_float2(0.f, 0.f);
+    if (e < nA_ops) {  // Aop[row, k] of slice row / nb
+      const uint64_t row = e / K, k = e % K, l = k >> 1, slice = row >> S.nB;
+      const uint64_t xb = spread(row & (nb - 1), S.b_bit, S.nB);
+      const float2 z = l < L ? B[xb + (l << S.nB) + (slice << (S.nB + S.t))] : make_float2(0.f, 0.f);
       v = (k & 1) ? z.y : z.x;
-      const uint64_t rt = xb / kRows, kc = k / kKc;
+      const uint64_t rt = row / kRows, kc = k / kKc;
       dst = aimg + (rt * kch + kc) * 2 * kABlock;
       blk = kABlock;
-      const uint32_t o = blk_off((uint32_t)(xb % kRows), (uint32_t)(k % kKc));
+      const uint32_t o = blk_off((uint32_t)(row % kRows), (uint32_t)(k % kKc));
       const float h = tf32_rn(v);
       *reinterpret_cast<float *>(dst + o) = h;
       *reinterpret_cast<float *>(dst + blk + o) = tf32_rn(v - h);
-    } else {  // Bop[n, k], n = 2 x_A + o
-      const uint64_t f = e - nA_ops, n = f / K, k = f % K, l = k >> 1;
-      const uint64_t xa = n >> 1;
-      const float2 z = l < L ? A[xa + (l << nA)] : make_float2(0.f, 0.f);
+    } else {  // Bop[n, k], n = 2 column + o, of slice column / na
+      const uint64_t f = e - nA_ops, n = f / K, k = f % K, l = k >> 1, slice = (n >> 1) >> S.nA;
+      const uint64_t xa = spread((n >> 1) & (na - 1), S.a_bit, S.nA);
+      const float2 z = l < L ? A[xa + (l << S.nA) + (slice << (S.nA + S.t))] : make_float2(0.f, 0.f);
       const bool im_out = n & 1, im_in = k & 1;
       v = !im_out ? (im_in ? -z.y : z.x) : (im_in ? z.x : z.y);
       const uint64_t ct = n / (2 * kCols), kc = k / kKc;
@@ -121,14 +132,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
 
 __global__ void __launch_bounds__(128, 2)
 outer_mma_kernel(const unsigned char *__restrict__ aimg, const unsigned char *__restrict__ bimg, int rtiles, int ctiles,
-                 int kch, int nA, float scale, float2 *__restrict__ out, int *err) {
+                 int kch, const OuterShape S, float2 scale, float2 *__restrict__ out, int *err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char *sm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char *sa = sm, *sb = sm + 2 * kABlock;
   __shared__ __align__(8) uint64_t load_bar, mma_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ int stop;
-  const int tid = threadIdx.x, warp = tid >> 5;
+  __shared__ uint64_t col_at[kCols], row_at[kRows];  // x_A of a tile's columns, x_B of its rows
+  const int tid = threadIdx.x, warp = tid >> 5, nA = S.nA;
+  col_at[tid] = spread(tid, S.a_bit, 7);
+  row_at[tid] = spread(tid, S.b_bit, 7);
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&load_bar)));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mma_bar)));
@@ -148,12 +162,17 @@ outer_mma_kernel(const unsigned char *__restrict__ aimg, const unsigned char *__
   const uint64_t ntiles = (uint64_t)rtiles * ctiles;
   for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const uint64_t rt = tile / ctiles, ct = tile % ctiles;
+    const uint64_t xa0 = spread(ct * kCols, S.a_bit, nA), xb0 = spread(rt * kRows, S.b_bit, S.nB);
+    // the slices that the tile's fixed bits select
+    uint64_t slice_a = 0, slice_b = 0;
+    for (int j = 0; j < S.fix_a; ++j) slice_a |= ((xb0 >> S.fix_a_by[j]) & 1ull) << j;
+    for (int j = 0; j < S.fix_b; ++j) slice_b |= ((xa0 >> S.fix_b_by[j]) & 1ull) << j;
     for (int kc = 0; kc < kch; ++kc) {
       if (tid == 0) {
         const uint32_t lb = smem_u32(&load_bar);
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(lb), "r"(kSmem) : "memory");
-        const unsigned char *ga = aimg + (rt * kch + kc) * 2 * kABlock;
-        const unsigned char *gb = bimg + (ct * kch + kc) * 2 * kBBlock;
+        const unsigned char *ga = aimg + ((slice_b * rtiles + rt) * kch + kc) * 2 * kABlock;
+        const unsigned char *gb = bimg + ((slice_a * ctiles + ct) * kch + kc) * 2 * kBBlock;
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                      ::"r"(smem_u32(sa)), "l"(ga), "r"(2 * kABlock), "r"(lb) : "memory");
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -200,8 +219,14 @@ outer_mma_kernel(const unsigned char *__restrict__ aimg, const unsigned char *__
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t taddr = tmem + ((uint32_t)(32 * warp) << 16);
     const int lane = tid & 31;
+    // the absorbed CZs' signs: the bits of x_A whose parity is this lane's row's sign
+    uint64_t sign_mask = 0;
+    for (int j = 0; j < S.signs; ++j)
+      sign_mask ^= (((xb0 + row_at[32 * warp + lane]) >> S.sign_b[j]) & 1ull) << S.sign_a[j];
+    const uint32_t sign_base = __popcll(sign_mask & xa0);
     float4 *stg = reinterpret_cast<float4 *>(sa) + warp * 256;
-    float2 *rows = out + (((rt * kRows + (uint64_t)(32 * warp)) << nA) + ct * kCols);
+    const bool neighbours = S.a_bit[0] == 0;
+    auto scaled = [&](uint32_t v) { return fmaf(__uint_as_float(v), scale.x, __uint_as_float(v) * scale.y); };
 #pragma unroll 1
     for (int c = 0; c < 256; c += 32) {
       uint32_t r[32];
@@ -215,17 +240,27 @@ outer_mma_kernel(const unsigned char *__restrict__ aimg, const unsigned char *__
           : "r"(taddr + (uint32_t)c)
           : "memory");
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      if (sign_mask) {
+#pragma unroll
+        for (int q = 0; q < 32; ++q)  // (column c / 2 + q / 2 of the tile)
+          r[q] ^= (sign_base + __popcll(sign_mask & col_at[c / 2 + q / 2])) << 31;
+      }
 #pragma unroll
       for (int q = 0; q < 8; ++q)
         stg[lane * 8 + (q ^ (lane & 7))] =
-            make_float4(__uint_as_float(r[4 * q]) * scale, __uint_as_float(r[4 * q + 1]) * scale,
-                        __uint_as_float(r[4 * q + 2]) * scale, __uint_as_float(r[4 * q + 3]) * scale);
+            make_float4(scaled(r[4 * q]), scaled(r[4 * q + 1]), scaled(r[4 * q + 2]), scaled(r[4 * q + 3]));
       __syncwarp();
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         const int row = 4 * q + (lane >> 3), ch = lane & 7;
         const float4 v = stg[row * 8 + (ch ^ (row & 7))];
-        *reinterpret_cast<float4 *>(rows + ((uint64_t)row << nA) + c / 2 + 2 * ch) = v;
+        float2 *const to = out + ((xb0 + row_at[32 * warp + row]) << nA) + xa0 + col_at[c / 2 + 2 * ch];
+        if (neighbours) {
+          *reinterpret_cast<float4 *>(to) = v;
+        } else {
+          to[0] = make_float2(v.x, v.y);
+          to[1ull << S.a_bit[0]] = make_float2(v.z, v.w);
+        }
       }
       __syncwarp();
     }
@@ -249,16 +284,17 @@ outer_mma_kernel(const unsigned char *__restrict__ aimg, const unsigned char *__
 
 }  // namespace
 
-bool outer_sum_tc_supported(int nA, int nB, int t) { return nA >= 7 && nB >= 7 && t >= 0 && t <= 20; }
+bool outer_sum_tc_supported(const OuterShape &S) { return S.a_free >= 7 && S.b_free >= 7 && S.t >= 0 && S.t <= 20; }
 
-size_t outer_sum_tc_scratch(int nA, int nB, int t) {
-  const uint64_t kch = ((2ull << t) + kKc - 1) / kKc;
-  return (size_t)(((1ull << nB) / kRows) * kch * 2 * kABlock + ((1ull << nA) / kCols) * kch * 2 * kBBlock);
+size_t outer_sum_tc_scratch(const OuterShape &S) {
+  const uint64_t kch = ((2ull << S.t) + kKc - 1) / kKc;
+  return (size_t)((((1ull << S.nB) << S.fix_b) / kRows) * kch * 2 * kABlock +
+                  (((1ull << S.nA) << S.fix_a) / kCols) * kch * 2 * kBBlock);
 }
 
-cudaError_t launch_outer_sum_tc(const float2 *A, int nA, const float2 *B, int nB, int t, float scale, float2 *out,
+cudaError_t launch_outer_sum_tc(const float2 *A, const float2 *B, const OuterShape &S, float2 scale, float2 *out,
                                 void *scratch, int *err, cudaStream_t st) {
-  if (!outer_sum_tc_supported(nA, nB, t)) return cudaErrorInvalidValue;
+  if (!outer_sum_tc_supported(S)) return cudaErrorInvalidValue;
   static bool configured = false;
   if (!configured) {
     const cudaError_t e =
@@ -266,21 +302,21 @@ cudaError_t launch_outer_sum_tc(const float2 *A, int nA, const float2 *B, int nB
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  const int kch = (int)(((2ull << t) + kKc - 1) / kKc);
-  const int rtiles = (int)((1ull << nB) / kRows), ctiles = (int)((1ull << nA) / kCols);
+  const int kch = (int)(((2ull << S.t) + kKc - 1) / kKc);
+  const int rtiles = (int)((1ull << S.nB) / kRows), ctiles = (int)((1ull << S.nA) / kCols);
   unsigned char *aimg = static_cast<unsigned char *>(scratch);
-  unsigned char *bimg = aimg + (size_t)rtiles * kch * 2 * kABlock;
-  const uint64_t work = ((1ull << nB) + (2ull << nA)) * (uint64_t)kch * kKc;
+  unsigned char *bimg = aimg + ((size_t)rtiles << S.fix_b) * kch * 2 * kABlock;
+  const uint64_t work = (((1ull << S.nB) << S.fix_b) + ((2ull << S.nA) << S.fix_a)) * (uint64_t)kch * kKc;
   uint64_t pgrid = (work + 255) / 256;
   const uint64_t pmax = (uint64_t)device_sm_count() * 8;
   if (pgrid > pmax) pgrid = pmax;
-  outer_prep_kernel<<<(unsigned)pgrid, 256, 0, st>>>(A, nA, B, nB, t, kch, aimg, bimg);
+  outer_prep_kernel<<<(unsigned)pgrid, 256, 0, st>>>(A, B, S, kch, aimg, bimg);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   uint64_t grid = (uint64_t)device_sm_count() * 2;
   const uint64_t ntiles = (uint64_t)rtiles * ctiles;
   if (grid > ntiles) grid = ntiles;
-  outer_mma_kernel<<<(unsigned)grid, 128, kSmem + 1024, st>>>(aimg, bimg, rtiles, ctiles, kch, nA, scale, out, err);
+  outer_mma_kernel<<<(unsigned)grid, 128, kSmem + 1024, st>>>(aimg, bimg, rtiles, ctiles, kch, S, scale, out, err);
   return cudaGetLastError();
 }
 

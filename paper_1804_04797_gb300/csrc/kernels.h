@@ -65,17 +65,34 @@ int device_sm_count();
 // slice c of the branch bits n_cur..n_new-1 (they were |+> until now), in place.
 cudaError_t launch_fork(float2 *psi, int n_cur, int n_new, cudaStream_t st);
 
-// Full state from two batched half-states (Eqs. 6-7): out[x_A + (x_B << nA)] = scale *
-// sum_l A[x_A + (l << nA)] B[x_B + (l << nB)] over 2^t branches (fp32).
-// The same product on the tensor cores (TF32x3, k_outer_tc.cu): half states of >= 7
-// qubits; scratch: outer_sum_tc_scratch bytes of device memory for the operand images;
-// err: a device int set non-zero if a bounded wait gave up.
-bool outer_sum_tc_supported(int nA, int nB, int t);
-size_t outer_sum_tc_scratch(int nA, int nB, int t);
-cudaError_t launch_outer_sum_tc(const float2 *A, int nA, const float2 *B, int nB, int t, float scale, float2 *out,
-                                void *scratch, int *err, cudaStream_t st);
-cudaError_t launch_outer_sum(const float2 *A, int nA, const float2 *B, int nB, int t, float scale, float2 *out,
+// The product of two batched half-states (Eqs. 6-7): A holds 2^t summed branches (bits nA..)
+// and above them one bit per branch that a bit of x_B fixes, B likewise.
+struct OuterShape {
+  int nA = 0, nB = 0, t = 0;
+  // x_A's bits in the order of the tiles' columns: those that fix no branch of B (a_free of
+  // them, ascending), then those that do; x_B's likewise
+  int a_free = 0, b_free = 0;
+  uint8_t a_bit[34], b_bit[34];
+  // branch bit nA + t + j of A is bit fix_a_by[j] of x_B; nB + t + j of B bit fix_b_by[j] of x_A
+  int fix_a = 0, fix_b = 0;
+  uint8_t fix_a_by[34], fix_b_by[34];
+  // signs (-1)^{x_A bit sign_a[j] * x_B bit sign_b[j]} (crossing CZs that only sign the output)
+  int signs = 0;
+  uint8_t sign_a[64], sign_b[64];
+};
+
+// Full state from the halves: out[x_A + (x_B << nA)] = scale (hi + lo) * the signs * sum over the 2^t
+// branches l of A[x_A + (l << nA) + its slice] B[x_B + (l << nB) + its slice] (fp32).  At
+// most 2^30 tiles.
+cudaError_t launch_outer_sum(const float2 *A, const float2 *B, const OuterShape &shape, float2 scale, float2 *out,
                              cudaStream_t st);
+// The same product on the tensor cores (TF32x3, k_outer_tc.cu): at least 7 free bits in
+// either half; scratch: outer_sum_tc_scratch bytes of device memory for the operand images;
+// err: a device int set non-zero if a bounded wait gave up.
+bool outer_sum_tc_supported(const OuterShape &shape);
+size_t outer_sum_tc_scratch(const OuterShape &shape);
+cudaError_t launch_outer_sum_tc(const float2 *A, const float2 *B, const OuterShape &shape, float2 scale, float2 *out,
+                                void *scratch, int *err, cudaStream_t st);
 
 // <a|b> = sum conj(a_i) b_i of two 2^n states: out2 = (re, im), fp64 (partials: 2 *
 // reduce_partials_needed() doubles of scratch).
