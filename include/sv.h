@@ -350,7 +350,8 @@ sv_status sv_inner_product(sv_state *a, sv_state *b, double *out_re_im);
  * split_layer (U1 = layers 0..split_layer, the H layer included; U2 = the rest),
  * |psi> = U1 H^n |0> is computed once, and for every bitstring x, |phi_x> = U2^dagger |x>
  * and alpha_x = <phi_x|psi>; on plan-specialised kernels (sv_options.jit) the last pass
- * of phi_x sums <phi_x|psi> instead of storing phi_x.  Two n-qubit states are allocated
+ * of phi_x sums <phi_x|psi> instead of storing phi_x, and the passes before it run only
+ * where phi_x can differ from zero.  Two n-qubit states are allocated
  * (2 x 8 x 2^n bytes, at most n = 34 on GB300) and freed on return; out_re_im receives
  * 2m doubles.  A split_layer at or beyond the depth gives the plain amplitudes of the
  * full state. */

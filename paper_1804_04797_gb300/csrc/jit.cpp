@@ -410,6 +410,16 @@ int pipe_threads(const svp::Plan &P, int kpr, int pass, bool inner) {
   return G * (1 << (dp.m - 1 - kpr)) + 32 + (direct ? 0 : 32) + (pass_matrix_stages(P, pass) > 0 ? 32 : 0);
 }
 
+// The qubits on which pass `pass` may find amplitudes other than those of its starting basis
+// state: the tiles' qubits of the passes before it (every qubit for other plans).
+static uint64_t support(const svp::Plan &P, int pass) {
+  if (!P.basis) return ~0ull;
+  uint64_t u = 0;
+  for (int k = 0; k < pass; ++k)
+    for (int i = 0; i < P.passes[(size_t)k].m; ++i) u |= 1ull << P.passes[(size_t)k].tq[i];
+  return u;
+}
+
 std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) {
   const svp::DevPass &dp = P.passes[(size_t)pass];
   const int m = dp.m;
@@ -420,6 +430,32 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
   const bool init = (dp.flags & (svp::PF_INIT_UNIFORM | svp::PF_INIT_ZERO)) != 0;
   const bool last = (size_t)pass + 1 == P.passes.size();
   inner = inner && last;
+  // a plan from a basis state: the tile index bits that take both values (the others are
+  // x's), and whether tile qubits outside the support leave most of the tile zero -- the
+  // first stage then reads the rest itself, straight into its registers
+  const uint64_t U = support(P, pass);
+  uint64_t vary = 0;
+  bool masked = false;
+  for (int i = 0; i < dp.nt; ++i) vary |= ((U >> dp.ntq[i]) & 1ull) << i;
+  for (int i = 0; i < m; ++i) masked = masked || !((U >> dp.tq[i]) & 1ull);
+  const bool all_tiles = vary == (dp.nt >= 64 ? ~0ull : (1ull << dp.nt) - 1);
+  // C statements: this CTA's tile of turn `var` (leaves the loop after the last one)
+  auto tile_stmt = [&](const char *var) {
+    std::string t = std::string("const unsigned long long tile_") + (all_tiles ? "id" : "j") + " = tile_of<RUN>(" + var +
+                    ", num_tiles);\n      if (tile_" + (all_tiles ? "id" : "j") + " >= num_tiles) break;\n";
+    if (all_tiles) return t;
+    t += "      const unsigned long long tile_id = ba.fixed";
+    for (int i = 0, from = 0; i < dp.nt;) {
+      if (!((vary >> i) & 1ull)) { ++i; continue; }
+      int k = i;
+      while (k < dp.nt && ((vary >> k) & 1ull)) ++k;
+      t += " | (((tile_j >> " + std::to_string(from) + ") & " + std::to_string((1ull << (k - i)) - 1) + "ull) << " +
+           std::to_string(i) + ")";
+      from += k - i;
+      i = k;
+    }
+    return t + ";\n      (void)tile_id;\n";
+  };
   // the last stage's output: straight from registers (whole rows per quarter warp), or
   // back into the slot in memory order, written out by a storer warp with TMA stores
   const bool direct = inner || pipe_direct_store(P, pass);
@@ -457,7 +493,8 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
   }
   os << "\nextern \"C\" __global__ void __launch_bounds__(" << NT << ", 1)\nsv_pass"
      << "(float2 *__restrict__ psi, svk::DevPlanView plan, unsigned long long num_tiles, double *sums,\n"
-     << "        const float2 *__restrict__ other, const __grid_constant__ TmaDesc tmap) {\n"
+     << "        const float2 *__restrict__ other, const __grid_constant__ TmaDesc tmap"
+     << (P.basis ? ", const svk::BasisArgs ba" : "") << ") {\n"
      << "  constexpr int G = " << G << ", S = " << S << ", TG = " << TG << ";\n"
      << "  constexpr int RUN = " << (mma ? 0 : tile_run_log()) << ";  // runs of 2^RUN neighbouring tiles per turn\n"
      << "  constexpr unsigned TILE_BYTES = " << (8u << m) << "u;\n"
@@ -514,14 +551,14 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
      << "    // producer warp: tile i of this CTA into slot i mod S once the slot is empty\n"
      << "    unsigned long long i = 0;\n"
      << "    for (;; ++i) {\n"
-     << "      const unsigned long long tile_id = tile_of<RUN>(i, num_tiles);\n"
-     << "      if (tile_id >= num_tiles) break;\n"
+     << "      " << tile_stmt("i")
      << "      const int s = (int)(i % S);\n"
      << "      bool ok = i < S || mbar_wait(&empty_bar[s], (uint32_t)((i / S - 1) & 1), kWaitNs);\n"
      << "      ok = __all_sync(0xffffffffu, ok);\n"
      << "      if (!ok) { if (lane == 0) atomicExch(plan.err, 3); break; }\n";
-  if (init) {
-    os << "      if (lane == 0) mbar_arrive(&full_bar[s]);  // generated tile: nothing to read\n";
+  if (init || masked) {
+    os << "      if (lane == 0) mbar_arrive(&full_bar[s]);  // "
+       << (init ? "generated tile: nothing to read" : "read by the first stage") << "\n";
   } else {
     os << "      if (lane == 0) mbar_arrive_tx(&full_bar[s], TILE_BYTES);\n"
        << "      __syncwarp();\n"
@@ -534,7 +571,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
        << "      }\n";
   }
   os << "    }\n";
-  if (!init)
+  if (!init && !masked)
     os << "    // every issued copy has landed before the CTA exits (bounded)\n"
        << "    for (unsigned long long k = i > (unsigned long long)S ? i - S : 0; k < i; ++k)\n"
        << "      mbar_wait(&full_bar[k % S], (uint32_t)((k / S) & 1), kWaitNs);\n";
@@ -597,8 +634,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
        << "    // storer warp: tile i out of its slot once its group has written it back, then\n"
        << "    // the slot goes to the producer\n"
        << "    for (unsigned long long i = 0;; ++i) {\n"
-       << "      const unsigned long long tile_id = tile_of<RUN>(i, num_tiles);\n"
-       << "      if (tile_id >= num_tiles) break;\n"
+       << "      " << tile_stmt("i")
        << "      const int s = (int)(i % S);\n"
        << "      bool ok = mbar_wait(&done_bar[s], (uint32_t)((i / S) & 1), kWaitNs);\n"
        << "      ok = __all_sync(0xffffffffu, ok);\n"
@@ -791,8 +827,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
        << "    const int g = tid / TG, t = tid % TG;\n"
        << "    const int bar_id = 1 + g;\n"
        << "    for (unsigned long long i = g;; i += G) {\n"
-       << "      const unsigned long long tile_id = tile_of<RUN>(i, num_tiles);\n"
-       << "      if (tile_id >= num_tiles) break;\n"
+       << "      " << tile_stmt("i")
        << "      const int slot = (int)(i % S);\n"
        << "      const bool ok = mbar_wait(&full_bar[slot], (uint32_t)((i / S) & 1), kWaitNs);\n"
        << "      if (group_any(bar_id, TG, !ok)) { if (t == 0) atomicExch(plan.err, 3); break; }\n"
@@ -814,8 +849,35 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
         os << (j ? ", " : "") << hex32(P.gtab[(size_t)svp::kGroupEntries * si + svp::kRegEntry + j].L);
       os << "};\n      Regs R, I;\n      int ph = 0;\n      bool zero = false;\n"
          << "      const uint32_t a0 = " << group_expr(P, si, "t", false) << ";\n";
-      if (s == 0 && init) os << "      init_regs(R, I, P, W);\n";
-      else os << "      load_group_rx<" << (s == 0 ? "true" : "false") << ">(tile, a0, rx, R, I);\n";
+      if (s == 0 && init) {
+        os << "      init_regs(R, I, P, W);\n";
+      } else if (s == 0 && masked) {
+        // zero where a tile bit outside the support is not x's
+        uint32_t gm = 0, pm = 0;
+        for (int i = 0; i < m - 1 - kpr; ++i) gm |= (uint32_t)!((U >> dp.tq[st.nonr[i]]) & 1ull) << i;
+        for (int j = 0; j < kpr; ++j) pm |= (uint32_t)!((U >> dp.tq[st.rbit[j]]) & 1ull) << j;
+        os << "      const bool mine = ((uint32_t)t & " << hex32(gm) << ") == ba.group;\n";
+        if (U == 0) {  // |x> itself
+          os << "#pragma unroll\n      for (int p = 0; p < kP; ++p) {\n"
+             << "        const bool hit = mine && (ba.regs & 255u) == (uint32_t)p;\n"
+             << "        R[p] = f2(hit && !(ba.regs & 256u) ? 1.f : 0.f, hit && (ba.regs & 256u) ? 1.f : 0.f);\n"
+             << "        I[p] = f2(0.f, 0.f);\n      }\n";
+        } else {
+          os << "      {\n      const unsigned long long g0 = base + (" << group_expr(P, si, "t", true) << ");\n"
+             << "      const unsigned long long o0[" << (1 << kpr) << "] = {";
+          for (int p = 0; p < (1 << kpr); ++p) {
+            uint64_t off = 0;
+            for (int j = 0; j < kpr; ++j)
+              if ((p >> j) & 1) off ^= P.gtab[(size_t)svp::kGroupEntries * si + svp::kRegEntry + j].G;
+            os << (p ? ", " : "") << off << "ull";
+          }
+          os << "};\n#pragma unroll\n      for (int p = 0; p < kP; ++p) {\n"
+             << "        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);\n"
+             << "        if (mine && ((uint32_t)p & " << hex32(pm) << ") == ba.regs)\n"
+             << "          x = __ldcg(reinterpret_cast<const float4 *>(psi + g0 + o0[p]));\n"
+             << "        R[p] = f2(x.x, x.z);\n        I[p] = f2(x.y, x.w);\n      }\n      }\n";
+        }
+      } else os << "      load_group_rx<" << (s == 0 ? "true" : "false") << ">(tile, a0, rx, R, I);\n";
       if (last_stage && direct)  // the slot is free once every thread of the group has read it
         os << "      fence_proxy_async();\n      mbar_arrive(&empty_bar[slot]);\n";
       emit_stage_ops(os, P, st, &pending, true);
@@ -1340,9 +1402,10 @@ cudaError_t prepare_passes(const Module *Mc, const svp::Plan &P) {
 
 unsigned max_pass_grid() { return (unsigned)svk::device_sm_count() * 32u; }  // <= 32 CTAs per SM
 
-cudaError_t launch_pass(const Module *Mc, float2 *psi, int n, const svk::DevPlanView &view, int pass,
-                        const svp::DevPass &hp, cudaStream_t st, double *sums, unsigned *grid_out,
-                        const float2 *other) {
+// One pass over `tiles` tiles; ba: a basis plan's arguments (else null).
+static cudaError_t launch_tiles(const Module *Mc, float2 *psi, int n, const svk::DevPlanView &view, int pass,
+                                const svp::DevPass &hp, uint64_t tiles, svk::BasisArgs *ba, cudaStream_t st, double *sums,
+                                unsigned *grid_out, const float2 *other) {
   Module *M = const_cast<Module *>(Mc);
   const Driver &D = driver();
   if (!D.ok || pass < 0 || pass >= (int)M->fn.size()) return cudaErrorInvalidValue;
@@ -1352,7 +1415,6 @@ cudaError_t launch_pass(const Module *Mc, float2 *psi, int n, const svk::DevPlan
   pass_shape(M, pass, m, &threads, &smem);
   if (!configure_pass(M, pass, m)) return cudaErrorLaunchFailure;
   CUfunction f = M->fn[pass];
-  const uint64_t tiles = 1ull << (n - m);
   uint64_t grid = (uint64_t)svk::device_sm_count() * (uint64_t)M->per_sm[pass];
   if (grid > tiles) grid = tiles;
   unsigned long long num_tiles = tiles;
@@ -1374,13 +1436,44 @@ cudaError_t launch_pass(const Module *Mc, float2 *psi, int n, const svk::DevPlan
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
-    void *args[] = {&psi, &v, &num_tiles, &sums, &other, &map};
+    void *args[] = {&psi, &v, &num_tiles, &sums, &other, &map, ba};
     r = D.launch(f, (unsigned)grid, 1, 1, (unsigned)threads, 1, 1, (unsigned)smem, (CUstream)st, args, nullptr);
   } else {
     void *args[] = {&psi, &v, &num_tiles, &sums, &other};
     r = D.launch(f, (unsigned)grid, 1, 1, (unsigned)threads, 1, 1, (unsigned)smem, (CUstream)st, args, nullptr);
   }
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorLaunchFailure;
+}
+
+cudaError_t launch_pass(const Module *M, float2 *psi, int n, const svk::DevPlanView &view, int pass,
+                        const svp::DevPass &hp, cudaStream_t st, double *sums, unsigned *grid_out,
+                        const float2 *other) {
+  return launch_tiles(M, psi, n, view, pass, hp, 1ull << (n - hp.m), nullptr, st, sums, grid_out, other);
+}
+
+cudaError_t launch_basis_pass(const Module *M, float2 *psi, const svk::DevPlanView &view, const svp::Plan &P, int pass,
+                              uint64_t x, cudaStream_t st, double *sums, unsigned *grid_out, const float2 *other,
+                              double *bytes) {
+  const svp::DevPass &hp = P.passes[(size_t)pass];
+  if (!pass_is_pipelined(P, pass)) return cudaErrorInvalidValue;
+  const uint64_t U = support(P, pass);
+  svk::BasisArgs ba = {0, 0, 0};
+  int vary = 0, known = 0;  // tile index bits, tile bits, of the support
+  for (int i = 0; i < hp.nt; ++i) {
+    if ((U >> hp.ntq[i]) & 1ull) ++vary;
+    else ba.fixed |= ((x >> hp.ntq[i]) & 1ull) << i;
+  }
+  for (int i = 0; i < hp.m; ++i) known += (int)((U >> hp.tq[i]) & 1ull);
+  const svp::DevStage &s0 = P.stages[hp.stage_begin];
+  auto bit = [&](int tile_bit) -> uint32_t {
+    const int q = hp.tq[tile_bit];
+    return ((U >> q) & 1ull) ? 0u : (uint32_t)((x >> q) & 1ull);
+  };
+  for (int i = 0; i < hp.m - 1 - M->kpr; ++i) ba.group |= bit(s0.nonr[i]) << i;
+  for (int j = 0; j < M->kpr; ++j) ba.regs |= bit(s0.rbit[j]) << j;
+  ba.regs |= bit(0) << 8;
+  if (bytes) *bytes = 8.0 * (double)(1ull << vary) * ((double)(1ull << hp.m) + (U ? (double)(1ull << known) : 0.0));
+  return launch_tiles(M, psi, P.n, view, pass, hp, 1ull << vary, &ba, st, sums, grid_out, other);
 }
 
 }  // namespace svj

@@ -76,6 +76,10 @@ struct Plan {
   // plan kernels of a fused packed plan: its matrix stages run on the tensor cores
   // (0 = none, 1 = F16x3, 2 = TF32x3; B operands in `mats`, set with the plan's matrices)
   int mma = 0;
+  // plan kernels that start from a basis state |x> without writing it (x a launch argument):
+  // pass k runs the tiles that hold non-zero amplitudes only -- outside the qubits of the
+  // tiles before it the state is still x -- and reads none that no pass has written
+  bool basis = false;
 };
 
 // Build the plan.  fresh_state: the state is |0..0> and was never written, so a

@@ -145,4 +145,12 @@ struct DevPlanView {
   const svp::DevGroupEntry *gtab;  // kGroupEntries group-addressing entries per stage
 };
 
+// Where a pass of a plan that starts from the basis state |x> finds x (Plan::basis): x's bits
+// at the tile-index positions outside the support, at the first stage's group bits and at
+// its register slots (bit 8: the pack bit) outside it.
+struct BasisArgs {
+  uint64_t fixed;
+  uint32_t group, regs;
+};
+
 }  // namespace svk
