@@ -82,7 +82,7 @@ static void interp_shape(const sv_options &o, int n, svp::Options *po) {
   }
 }
 
-svp::Options apply_plan_options(const sv_options &o, int n, bool *want_jit) {
+svp::Options apply_plan_options(const sv_options &o, int n, bool *want_jit, bool one_shape) {
   svp::Options po = plan_options(o);
   // tensor cores on the pipelined plan kernels (the default for 5-qubit blocks on
   // 12-qubit tiles): a fused packed plan -- stages of tile bit 0 and four register slots,
@@ -118,7 +118,7 @@ svp::Options apply_plan_options(const sv_options &o, int n, bool *want_jit) {
     const int m = std::min(po.m, n);
     if (o.pipeline >= 0 && po.c == 4 && m >= 10 && m <= 13) po.layout = 1;
   }
-  if (!*want_jit && !po.fused) interp_shape(o, n, &po);
+  if (!*want_jit && !po.fused && !one_shape) interp_shape(o, n, &po);
   return po;
 }
 
@@ -573,7 +573,7 @@ sv_status apply_gates(sv_state *s, const std::vector<svp::Gate> &g) {
   svp::Plan P;
   const char *err = nullptr;
   bool want_jit = false;
-  svp::Options po = apply_plan_options(s->opts, s->n, &want_jit);
+  svp::Options po = apply_plan_options(s->opts, s->n, &want_jit, s->one_shape);
   PlainTune tune;
   if (s->opts.autotune == 1 && want_jit && !po.fused && po.layout == 1 && s->fresh && s->opts.tile_bits == 0) {
     if ((st = autotune_plain(s, g, po, &tune)) != SV_OK) return st;

@@ -185,6 +185,7 @@ sv_status run_branch_tree(sv_state *full, int n_base, const std::vector<svp::Gat
     view.opts = full->opts;
     view.stream = full->stream;
     view.device = full->device;
+    view.one_shape = full->one_shape;
     view.fresh = first;
     view.user_writes = true;
     const sv_status st = apply_gates(&view, seg);
@@ -260,6 +261,7 @@ extern "C" sv_status sv_branch_amplitudes(const sv_lattice *lat, const sv_cut *c
   Holder A, B;
   if ((st = sv_create(na + C.ta, &o, &A.s)) != SV_OK) return st;
   if ((st = sv_create(nb + C.tb, &o, &B.s)) != SV_OK) return st;
+  A.s->one_shape = B.s->one_shape = true;
   if ((st = run_branch_tree(A.s, na, C.ga)) != SV_OK) return st;
   if ((st = run_branch_tree(B.s, nb, C.gb)) != SV_OK) return st;
   if (m == 0) return SV_OK;
@@ -368,9 +370,11 @@ extern "C" sv_status sv_amplitudes_by_inner_product(const sv_lattice *lat, int s
   if (opts) o = *opts;
   Holder A, B;
   if ((st = sv_create(n, &o, &A.s)) != SV_OK) return st;
+  A.s->one_shape = true;
   if ((st = sv_apply_circuit(A.s, g1.data(), g1.size())) != SV_OK) return st;  // |psi> = U1 H|0>
   if (m == 0) return SV_OK;
   if ((st = sv_create(n, &o, &B.s)) != SV_OK) return st;
+  B.s->one_shape = true;
   std::vector<svp::Gate> g2_inv;
   if ((st = convert_gates(n, g2.data(), g2.size(), true, &g2_inv)) != SV_OK) return st;
   bool done = false;

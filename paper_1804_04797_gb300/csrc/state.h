@@ -24,6 +24,10 @@ struct sv_state {
   int device = 0;
   bool fresh = false;     // logically |0..0> but not yet written (lazy initial state)
   bool broken = false;    // an apply failed part-way: content undefined
+  // a state of a few-amplitude call (cut branches, inner products): plans on the interpreting
+  // kernel keep one shape, so that an amplitude does not change, to the last bit, with the
+  // tuning of the state path's shapes (interp_shape)
+  bool one_shape = false;
   // device scratch: packed plan, gather/reduction buffers
   void *d_plan = nullptr;
   size_t d_plan_cap = 0;
@@ -78,7 +82,7 @@ sv_status ensure_device_buffer(void **buf, size_t *cap, size_t need);
 svp::Options plan_options(const sv_options &o);
 // The plan options sv_apply_circuit uses for an n-qubit state; *want_jit: the plain path
 // is to run on plan-specialised kernels.
-svp::Options apply_plan_options(const sv_options &o, int n, bool *want_jit);
+svp::Options apply_plan_options(const sv_options &o, int n, bool *want_jit, bool one_shape = false);
 sv_status check_options(const sv_options &o);
 sv_status convert_gates(int n, const sv_gate *g, size_t count, bool inverse, std::vector<svp::Gate> *out);
 // The plan's device copy (in s->d_plan): as the plan kernels read it, or (interp) as the
