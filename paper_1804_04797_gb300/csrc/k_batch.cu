@@ -1,7 +1,7 @@
 // K7: the uneven batch in one persistent launch.
 //
-// Every CTA repeatedly takes the next item (one tile of one pass of one circuit) from a
-// global counter and runs the plain tile pass on it.  Before an item of pass p it waits
+// Every CTA repeatedly takes the next item (a run of tiles of one pass of one circuit) from a
+// global counter and runs the plain tile pass on them.  Before an item of pass p it waits
 // until every tile of pass p-1 of the same circuit is done (a per-circuit-pass counter),
 // with a bounded spin: a wait that gives up sets the error word and the CTA leaves.  The
 // queue holds all circuits' first passes, then all second passes, ..., so the waits are
@@ -35,7 +35,7 @@ __device__ __forceinline__ unsigned int load_acquire(const unsigned int *p) {
 
 __global__ void __launch_bounds__(256, 2)
 batch_kernel(float2 *__restrict__ states, const unsigned char *__restrict__ blocks, const BatchCP *__restrict__ cps,
-             const BatchItem *__restrict__ items, uint64_t n_items, unsigned int *words, uint32_t tile_bytes,
+             const BatchItem *__restrict__ items, uint32_t n_items, unsigned int *words, uint32_t tile_bytes,
              unsigned long long wait_ns) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4 *tile = reinterpret_cast<float4 *>(smem_raw);
@@ -59,27 +59,52 @@ batch_kernel(float2 *__restrict__ states, const unsigned char *__restrict__ bloc
     if (it.cp != cur_cp) {
       fetch_block(blk, src, cp.block_bytes);
       cur_cp = it.cp;
-    }
-    if (tid == 0 && cp.prev != kNoPrev) {
-      const unsigned int need = cps[cp.prev].tiles;
-      if (load_acquire(&done[cp.prev]) < need) {
-        const unsigned long long t0 = now_ns();
-        while (load_acquire(&done[cp.prev]) < need) {
-          if (now_ns() - t0 > wait_ns) {
-            atomicExch(&words[1], 1u);
-            s_stop = 1;
-            break;
+      if (tid == 0 && cp.prev != kNoPrev) {
+        const unsigned int need = cps[cp.prev].tiles;
+        if (load_acquire(&done[cp.prev]) < need) {
+          const unsigned long long t0 = now_ns();
+          while (load_acquire(&done[cp.prev]) < need) {
+            if (now_ns() - t0 > wait_ns) {
+              atomicExch(&words[1], 1u);
+              s_stop = 1;
+              break;
+            }
           }
         }
       }
     }
     __syncthreads();
     if (s_stop) break;
-    process_tile<kBatchSlots>(states + cp.state_off, blk, src, tile, it.tile);
+    const uint32_t end = min(it.tile + (1u << cp.run), cp.tiles);
+    for (uint32_t t = it.tile; t < end; ++t) {
+      if (t != it.tile) __syncthreads();  // the tile before has been read
+      process_tile<kBatchSlots>(states + cp.state_off, blk, src, tile, t);
+    }
     __threadfence();  // each thread's stores visible device-wide before the count
     __syncthreads();
-    if (tid == 0) atomicAdd(&done[it.cp], 1u);
+    if (tid == 0) atomicAdd(&done[it.cp], end - it.tile);
   }
+}
+
+__global__ void pick_kernel(const float2 *__restrict__ psi, const __grid_constant__ PickArgs args, int count,
+                            float2 *__restrict__ out) {
+  const int i = threadIdx.x;
+  if (i < count) out[i] = psi[args.index[i]];
+}
+
+// The queue, written where it is read: built by the host it took 0.48 ms of a call on 64 new
+// circuits of 10..22 qubits (137 k items, one push each, and their copy).
+__global__ void items_kernel(const BatchCP *__restrict__ cps, uint32_t n_cps, BatchItem *__restrict__ items,
+                             uint32_t n_items) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n_items) return;
+  uint32_t at = 0, end = n_cps;  // the last circuit-pass that starts at or before the item
+  while (end - at > 1) {
+    const uint32_t mid = at + (end - at) / 2;
+    if (cps[mid].first <= i) at = mid;
+    else end = mid;
+  }
+  items[i] = BatchItem{at, (i - cps[at].first) << cps[at].run};
 }
 
 __device__ __forceinline__ double warp_sum(double x) {
@@ -146,26 +171,60 @@ __global__ void batch_stats_final(const double *partials, const int *chunk_begin
 
 int batch_block_threads(int m) { return 1 << (m - 1 - kBatchSlots); }
 
-cudaError_t launch_batch(float2 *states, const unsigned char *blocks, uint32_t max_block_bytes, const BatchCP *cps,
-                         const BatchItem *items, uint64_t n_items, unsigned int *words, int m, cudaStream_t st,
-                         unsigned long long wait_ns, int max_grid) {
+namespace {
+size_t batch_smem(uint32_t max_block_bytes, int m) {
+  return (sizeof(float2) << m) + svp::interp_smem_max(max_block_bytes) + svp::kInterpPad;
+}
+}  // namespace
+
+// An item's fixed cost -- the counter, the item, the pass's program, the dependency, the fence
+// and the count -- is shared by its tiles, but a pass ends with the last of its items, so the
+// runs grow with the tiles that every CTA has to take (us at runs of 1 / 2 / 4 / 8 / 16 tiles):
+//   40 circuits of 8..10 qubits 61 / 77 / 111 / 109 / 109, 84 of 11..18 190 / 224 / 353 / 520 / 757,
+//   512 of 12..16 403 / 411 / 450 / 570 / 860, 64 of 10..22 1265 / 1249 / 1304 / 1445 / 2002,
+//   96 of 14..22 1913 / 1834 / 1810 / 1805 / 1920, 256 of 16..23 12837 / 12362 / 12167 / 12083 / 12055.
+// A small circuit's pass keeps 64 items.
+int batch_run_log(uint32_t tiles, double per_cta) {
+  int run = 0;
+  while (run < 4 && per_cta >= 16 << run && tiles >= 128u << run) ++run;
+  return run;
+}
+
+int batch_grid(uint32_t max_block_bytes, int m) {
   static bool configured = false;
   if (!configured) {  // tiles of <= 13 qubits (capi_batch)
-    cudaError_t e = cudaFuncSetAttribute(
-        batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-        (int)((sizeof(float2) << 13) + svp::kInterpResident + svp::kInterpPad));
-    if (e != cudaSuccess) return e;
+    if (cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)batch_smem(svp::kInterpResident, 13)) != cudaSuccess)
+      return 0;
     configured = true;
   }
-  const size_t tile_bytes = sizeof(float2) << m;
-  const size_t smem = tile_bytes + svp::interp_smem_max(max_block_bytes) + svp::kInterpPad;
-  const int threads = batch_block_threads(m);
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel, threads, smem);
-  if (e != cudaSuccess) return e;
-  int grid = device_sm_count() * (per_sm < 1 ? 1 : per_sm);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel, batch_block_threads(m),
+                                                    batch_smem(max_block_bytes, m)) != cudaSuccess)
+    return 0;
+  return device_sm_count() * (per_sm < 1 ? 1 : per_sm);
+}
+
+cudaError_t launch_batch(float2 *states, const unsigned char *blocks, uint32_t max_block_bytes, const BatchCP *cps,
+                         const BatchItem *items, uint32_t n_items, unsigned int *words, int m, cudaStream_t st,
+                         unsigned long long wait_ns, int max_grid) {
+  int grid = batch_grid(max_block_bytes, m);
+  if (grid < 1) return cudaGetLastError();
   if (max_grid > 0 && grid > max_grid) grid = max_grid;
-  batch_kernel<<<grid, threads, smem, st>>>(states, blocks, cps, items, n_items, words, (uint32_t)tile_bytes, wait_ns);
+  batch_kernel<<<grid, batch_block_threads(m), batch_smem(max_block_bytes, m), st>>>(
+      states, blocks, cps, items, n_items, words, (uint32_t)(sizeof(float2) << m), wait_ns);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_pick(const float2 *psi, const PickArgs &args, int count, float2 *out, cudaStream_t st) {
+  if (count < 1 || count > kPickMost) return cudaErrorInvalidValue;
+  pick_kernel<<<1, (count + 31) / 32 * 32, 0, st>>>(psi, args, count, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_batch_items(const BatchCP *cps, uint32_t n_cps, BatchItem *items, uint32_t n_items,
+                               cudaStream_t st) {
+  items_kernel<<<(n_items + 255) / 256, 256, 0, st>>>(cps, n_cps, items, n_items);
   return cudaGetLastError();
 }
 
