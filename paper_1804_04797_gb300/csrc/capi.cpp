@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -639,60 +640,60 @@ sv_status apply_gates(sv_state *s, const std::vector<svp::Gate> &g) {
   return SV_OK;
 }
 
-sv_status basis_inner_products(sv_state *s, const std::vector<svp::Gate> &g, const uint64_t *xs, size_t m,
-                               const sv_state *with, double *out, bool *done) {
+sv_status basis_inner_products(sv_state *with, const std::vector<svp::Gate> &g, const uint64_t *xs, size_t m,
+                               double *out, bool *done) {
   *done = false;
   sv_status st;
-  if ((st = set_device(s)) != SV_OK) return st;
-  if (s->opts.precision != SV_PREC_PLAIN || s->n < 6 || g.empty() || m == 0 || !s->owns) return SV_OK;
+  if ((st = set_device(with)) != SV_OK) return st;
+  if (with->opts.precision != SV_PREC_PLAIN || with->n < 6 || g.empty() || m == 0) return SV_OK;
   bool want_jit = false;
-  svp::Options po = apply_plan_options(s->opts, s->n, &want_jit);
+  svp::Options po = apply_plan_options(with->opts, with->n, &want_jit);
   if (!want_jit || po.fused || po.layout != 1) return SV_OK;
   svp::Plan P;
   const char *err = nullptr;
-  if (!svp::build_plan(s->n, g, po, false, &P, &err)) return fail(SV_ERR_ARG, err ? err : "planning failed");
+  if (!svp::build_plan(with->n, g, po, false, &P, &err)) return fail(SV_ERR_ARG, err ? err : "planning failed");
   P.basis = true;
   for (size_t p = 0; p < P.passes.size(); ++p)
     if (!svj::pass_is_pipelined(P, (int)p)) return SV_OK;
   std::string jerr;
   const svj::Module *M = svj::get_module(P, po.rk, &jerr, true);
   if (!M) return SV_OK;  // no compiler: the caller applies and reduces separately
-  s->plan_valid = false;
-  s->sums_valid = false;
+  // the backward states' handle, with the memory of their support
+  struct Destroy {
+    void operator()(sv_state *b) const { sv_destroy(b); }
+  };
+  std::unique_ptr<sv_state, Destroy> back(new sv_state());
+  sv_state *s = back.get();
+  s->n = with->n;
+  s->owns = true;
+  s->opts = with->opts;
+  s->stream = with->stream;
+  s->device = with->device;
+  if (cudaMalloc(reinterpret_cast<void **>(&s->psi), sizeof(float2) << svj::basis_state_bits(P)) != cudaSuccess ||
+      cudaMalloc(reinterpret_cast<void **>(&s->d_sums), (2 + 2 * (size_t)svj::max_pass_grid()) * sizeof(double)) !=
+          cudaSuccess) {
+    cudaGetLastError();
+    return fail(SV_ERR_OOM, "allocation of the backward states failed");
+  }
   svk::DevPlanView view;
   if ((st = upload_plan(s, P, &view)) != SV_OK) return st;
-  if (!s->d_sums) {
-    if (cudaMalloc(&s->d_sums, (2 + 2 * (size_t)svj::max_pass_grid()) * sizeof(double)) != cudaSuccess) {
-      cudaGetLastError();
-      s->d_sums = nullptr;
-      return fail(SV_ERR_OOM, "sums buffer allocation failed");
-    }
-  }
   if ((st = ensure_device_buffer(&s->d_scratch, &s->d_scratch_cap, 2 * m * sizeof(double))) != SV_OK) return st;
   double *const d_out = static_cast<double *>(s->d_scratch);
-  // the other state's pending work first (the handles may use different streams)
-  cudaError_t e = with->stream == s->stream ? cudaSuccess : cudaStreamSynchronize(with->stream);
+  cudaError_t e = cudaSuccess;
   for (size_t j = 0; e == cudaSuccess && j < m; ++j) {
     unsigned grid = 0;
     for (size_t p = 0; e == cudaSuccess && p < P.passes.size(); ++p) {
       const bool last = p + 1 == P.passes.size();
-      double bytes = 0;
-      prof_begin(s);
       e = svj::launch_basis_pass(M, s->psi, view, P, (int)p, xs[j], s->stream, last ? s->d_sums + 2 : nullptr,
-                                 last ? &grid : nullptr, last ? with->psi : nullptr, &bytes);
-      prof_end(s, bytes);
-      if (s->prof) s->jit_launches += 1;
+                                 last ? &grid : nullptr, last ? with->psi : nullptr);
     }
     if (e == cudaSuccess) e = svk::launch_norm_final(s->d_sums + 2, (int)grid, d_out + 2 * j, s->stream);
-    if (s->prof) s->other_launches += 1;
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(out, d_out, 2 * m * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-  s->broken = true;  // the state is no circuit's result: its passes skipped what is zero
   if (e != cudaSuccess) return cuda_fail(e, "inner product pass");
   s->err_pending = view.err;
   if ((st = take_pending_error(s)) != SV_OK) return st;
-  if (s->prof) s->d2h += 2 * m * sizeof(double);
   *done = true;
   return SV_OK;
 }

@@ -373,12 +373,12 @@ extern "C" sv_status sv_amplitudes_by_inner_product(const sv_lattice *lat, int s
   A.s->one_shape = true;
   if ((st = sv_apply_circuit(A.s, g1.data(), g1.size())) != SV_OK) return st;  // |psi> = U1 H|0>
   if (m == 0) return SV_OK;
-  if ((st = sv_create(n, &o, &B.s)) != SV_OK) return st;
-  B.s->one_shape = true;
   std::vector<svp::Gate> g2_inv;
   if ((st = convert_gates(n, g2.data(), g2.size(), true, &g2_inv)) != SV_OK) return st;
   bool done = false;
-  if ((st = basis_inner_products(B.s, g2_inv, bits, m, A.s, out_re_im, &done)) != SV_OK || done) return st;
+  if ((st = basis_inner_products(A.s, g2_inv, bits, m, out_re_im, &done)) != SV_OK || done) return st;
+  if ((st = sv_create(n, &o, &B.s)) != SV_OK) return st;
+  B.s->one_shape = true;
   for (size_t j = 0; j < m; ++j) {
     // |phi_x> = U2^dagger |x>;  alpha_x = <phi_x|psi>: on plan kernels the last pass of
     // phi_x sums the inner product instead of storing phi_x

@@ -223,10 +223,39 @@ void emit_stage_end(std::ostringstream &os, int *pending, bool last_of_pass) {
   os << "      end_stage(R, I, " << now << ", ph, zero);\n";
 }
 
+// The qubits on which pass `pass` may find amplitudes other than those of its starting basis
+// state: the tiles' qubits of the passes before it (every qubit for other plans).
+uint64_t support(const svp::Plan &P, int pass) {
+  if (!P.basis) return ~0ull;
+  uint64_t u = 0;
+  for (int k = 0; k < pass; ++k)
+    for (int i = 0; i < P.passes[(size_t)k].m; ++i) u |= 1ull << P.passes[(size_t)k].tq[i];
+  return u;
+}
+
+// Where qubit q's bit lies in the state a plan's kernels address: a plan from a basis state
+// keeps the amplitudes its passes write and no others -- the support that its last pass, which
+// stores nothing, finds -- in index order (-1: not a bit of it).
+int place(const svp::Plan &P, int q) {
+  if (!P.basis) return q;
+  const uint64_t U = support(P, (int)P.passes.size() - 1);
+  return (U >> q) & 1ull ? __builtin_popcountll(U & ((1ull << q) - 1)) : -1;
+}
+uint64_t placed(const svp::Plan &P, uint64_t index) {
+  if (!P.basis) return index;
+  uint64_t v = 0;
+  for (; index; index &= index - 1) {
+    const int at = place(P, __builtin_ctzll(index));
+    if (at >= 0) v |= 1ull << at;
+  }
+  return v;
+}
+
 // C expression of a stage's group addressing for thread index `var`: the XOR over its
 // group-index bits of the stage's per-bit offsets (L: shared-memory byte offset, 32-bit;
-// G: global index offset, 64-bit), as compile-time constants -- no table reads.
-std::string group_expr(const svp::Plan &P, uint32_t si, const char *var, bool global) {
+// G: global index offset, 64-bit; `whole`: in the whole state, where P's is kept compactly), as
+// compile-time constants -- no table reads.
+std::string group_expr(const svp::Plan &P, uint32_t si, const char *var, bool global, bool whole = false) {
   const svp::DevStage &st = P.stages[si];
   (void)st;
   const svp::DevGroupEntry *ge = &P.gtab[(size_t)svp::kGroupEntries * si];
@@ -234,7 +263,7 @@ std::string group_expr(const svp::Plan &P, uint32_t si, const char *var, bool gl
   for (int i = 0; i < 12; ++i) {
     // bit i of the group index is entry (1 << (i % 4)) of table i / 4
     const svp::DevGroupEntry &x = ge[16 * (i / 4) + (1 << (i % 4))];
-    const uint64_t v = global ? x.G : (uint64_t)x.L;
+    const uint64_t v = !global ? (uint64_t)x.L : whole ? x.G : placed(P, x.G);
     if (!v) continue;
     char b[96];
     if (global) std::snprintf(b, sizeof(b), "((%s >> %d) & 1 ? 0x%llxull : 0ull)", var, i, (unsigned long long)v);
@@ -245,15 +274,18 @@ std::string group_expr(const svp::Plan &P, uint32_t si, const char *var, bool gl
 }
 
 // C expression of the global index of tile `tile_id`'s element 0: the tile index bits
-// spread over the non-tile qubits, one shift-and-mask per run of consecutive qubits.
-std::string tile_base_expr(const svp::DevPass &dp, const char *var = "tile_id") {
+// spread over the non-tile qubits, one shift-and-mask per run of consecutive qubits.  (whole: in
+// the whole state, where P's is kept compactly)
+std::string tile_base_expr(const svp::Plan &P, const svp::DevPass &dp, bool whole = false) {
   std::string e;
+  auto at = [&](int i) { return whole ? (int)dp.ntq[i] : place(P, dp.ntq[i]); };
   for (int i = 0; i < dp.nt;) {
     int j = i + 1;
-    while (j < dp.nt && dp.ntq[j] == dp.ntq[j - 1] + 1) ++j;
+    if (at(i) < 0) { i = j; continue; }
+    while (j < dp.nt && at(j) == at(j - 1) + 1) ++j;
     char b[160];
-    std::snprintf(b, sizeof(b), "((%s >> %d) & 0x%llxull) << %d", var, i, (unsigned long long)((1ull << (j - i)) - 1),
-                  (int)dp.ntq[i]);
+    std::snprintf(b, sizeof(b), "((tile_id >> %d) & 0x%llxull) << %d", i, (unsigned long long)((1ull << (j - i)) - 1),
+                  at(i));
     e += (e.empty() ? "" : " | ") + std::string("(") + b + ")";
     i = j;
   }
@@ -410,16 +442,6 @@ int pipe_threads(const svp::Plan &P, int kpr, int pass, bool inner) {
   return G * (1 << (dp.m - 1 - kpr)) + 32 + (direct ? 0 : 32) + (pass_matrix_stages(P, pass) > 0 ? 32 : 0);
 }
 
-// The qubits on which pass `pass` may find amplitudes other than those of its starting basis
-// state: the tiles' qubits of the passes before it (every qubit for other plans).
-static uint64_t support(const svp::Plan &P, int pass) {
-  if (!P.basis) return ~0ull;
-  uint64_t u = 0;
-  for (int k = 0; k < pass; ++k)
-    for (int i = 0; i < P.passes[(size_t)k].m; ++i) u |= 1ull << P.passes[(size_t)k].tq[i];
-  return u;
-}
-
 std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) {
   const svp::DevPass &dp = P.passes[(size_t)pass];
   const int m = dp.m;
@@ -471,10 +493,10 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
   // matrix stage so that one tile's products run while the group works on the other
   const int X = pass_streams(P, pass), NSTR = G * X;
   const int MT0 = G * TG + 32 + (direct ? 0 : 32);  // first thread of the MMA warp
+  auto row_of = [&](int q) { return place(P, q) < 4 ? 0u : 1u << (place(P, q) - 4); };
   std::string boxrow;  // C statements: row += the row offset of box j
   for (int b = 0; b + 7 < m; ++b)
-    boxrow += "        if ((j >> " + std::to_string(b) + ") & 1) row += " + std::to_string(1u << (dp.tq[7 + b] - 4)) +
-              ";\n";
+    boxrow += "        if ((j >> " + std::to_string(b) + ") & 1) row += " + std::to_string(row_of(dp.tq[7 + b])) + ";\n";
   std::ostringstream os;
   os << "// pipelined tile-pass kernel of one pass of a plan\n#define SV_PACK_R " << kpr
      << "\n#include \"tile_pack.cuh\"\n#include \"tile_pipe.cuh\"\n"
@@ -562,7 +584,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
   } else {
     os << "      if (lane == 0) mbar_arrive_tx(&full_bar[s], TILE_BYTES);\n"
        << "      __syncwarp();\n"
-       << "      const int row0 = (int)((" << tile_base_expr(dp) << ") >> 4);\n"
+       << "      const int row0 = (int)((" << tile_base_expr(P, dp) << ") >> 4);\n"
        << "      unsigned char *dst = smem + s * TILE_BYTES;\n"
        << "      for (int j = lane; j < " << nbox << "; j += 32) {\n"
        << "        int row = row0;\n"
@@ -642,7 +664,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
        << "      bool ok = mbar_wait(&done_bar[s], (uint32_t)((i / S) & 1), kWaitNs);\n"
        << "      ok = __all_sync(0xffffffffu, ok);\n"
        << "      if (!ok) { if (lane == 0) atomicExch(plan.err, 3); break; }\n"
-       << "      const int row0 = (int)((" << tile_base_expr(dp) << ") >> 4);\n"
+       << "      const int row0 = (int)((" << tile_base_expr(P, dp) << ") >> 4);\n"
        << "      const unsigned char *src = smem + s * TILE_BYTES;\n"
        << "      for (int j = lane; j < " << nbox << "; j += 32) {\n"
        << "        int row = row0;\n"
@@ -793,7 +815,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
            << "        fence_proxy_async();\n        mbar_arrive(&done_bar[slot]);\n        }\n";
         return;
       }
-      os << "        const unsigned long long base = " << tile_base_expr(dp) << ";\n"
+      os << "        const unsigned long long base = " << tile_base_expr(P, dp) << ";\n"
          << "        const unsigned long long gb = base + (" << group_expr(P, si, "t", true) << ");\n"
          << "        const unsigned long long go[" << (1 << kpr) << "] = {";
       for (int p = 0; p < (1 << kpr); ++p) {
@@ -836,10 +858,11 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
        << "      if (group_any(bar_id, TG, !ok)) { if (t == 0) atomicExch(plan.err, 3); break; }\n"
        << "      float4 *tile = reinterpret_cast<float4 *>(smem + slot * TILE_BYTES);\n"
        << "      (void)tile;\n"
-       << "      const unsigned long long base = " << tile_base_expr(dp) << ";\n"
+       << "      const unsigned long long base = " << tile_base_expr(P, dp) << ";\n"
        << "      (void)base;\n"
        << "      const uint32_t W = ((uint32_t)tile_id << " << (m - 1 - kpr) << ") | (uint32_t)t;\n"
        << "      (void)W;\n";
+    if (inner) os << "      const unsigned long long other_base = " << tile_base_expr(P, dp, true) << ";\n";
     int pending = 0;
     const int ns = dp.stage_count;
     for (int s = 0; s < ns; ++s) {
@@ -872,7 +895,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
             uint64_t off = 0;
             for (int j = 0; j < kpr; ++j)
               if ((p >> j) & 1) off ^= P.gtab[(size_t)svp::kGroupEntries * si + svp::kRegEntry + j].G;
-            os << (p ? ", " : "") << off << "ull";
+            os << (p ? ", " : "") << placed(P, off) << "ull";
           }
           os << "};\n#pragma unroll\n      for (int p = 0; p < kP; ++p) {\n"
              << "        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);\n"
@@ -904,13 +927,14 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
         continue;
       }
       // straight from registers to HBM (pair p at its global index)
-      os << "      const unsigned long long gb = base + (" << group_expr(P, si, "t", true) << ");\n"
+      os << "      const unsigned long long gb = " << (inner ? "other_base" : "base") << " + ("
+         << group_expr(P, si, "t", true, inner) << ");\n"
          << "      const unsigned long long go[" << (1 << kpr) << "] = {";
       for (int p = 0; p < (1 << kpr); ++p) {
         uint64_t off = 0;
         for (int j = 0; j < kpr; ++j)
           if ((p >> j) & 1) off ^= P.gtab[(size_t)svp::kGroupEntries * si + svp::kRegEntry + j].G;
-        os << (p ? ", " : "") << off << "ull";
+        os << (p ? ", " : "") << (inner ? off : placed(P, off)) << "ull";
       }
       os << "};\n";
       if (inner) {
@@ -1455,18 +1479,16 @@ cudaError_t launch_pass(const Module *M, float2 *psi, int n, const svk::DevPlanV
 }
 
 cudaError_t launch_basis_pass(const Module *M, float2 *psi, const svk::DevPlanView &view, const svp::Plan &P, int pass,
-                              uint64_t x, cudaStream_t st, double *sums, unsigned *grid_out, const float2 *other,
-                              double *bytes) {
+                              uint64_t x, cudaStream_t st, double *sums, unsigned *grid_out, const float2 *other) {
   const svp::DevPass &hp = P.passes[(size_t)pass];
   if (!pass_is_pipelined(P, pass)) return cudaErrorInvalidValue;
   const uint64_t U = support(P, pass);
   svk::BasisArgs ba = {0, 0, 0};
-  int vary = 0, known = 0;  // tile index bits, tile bits, of the support
+  int vary = 0;  // tile index bits of the support
   for (int i = 0; i < hp.nt; ++i) {
     if ((U >> hp.ntq[i]) & 1ull) ++vary;
     else ba.fixed |= ((x >> hp.ntq[i]) & 1ull) << i;
   }
-  for (int i = 0; i < hp.m; ++i) known += (int)((U >> hp.tq[i]) & 1ull);
   const svp::DevStage &s0 = P.stages[hp.stage_begin];
   auto bit = [&](int tile_bit) -> uint32_t {
     const int q = hp.tq[tile_bit];
@@ -1475,8 +1497,13 @@ cudaError_t launch_basis_pass(const Module *M, float2 *psi, const svk::DevPlanVi
   for (int i = 0; i < hp.m - 1 - M->kpr; ++i) ba.group |= bit(s0.nonr[i]) << i;
   for (int j = 0; j < M->kpr; ++j) ba.regs |= bit(s0.rbit[j]) << j;
   ba.regs |= bit(0) << 8;
-  if (bytes) *bytes = 8.0 * (double)(1ull << vary) * ((double)(1ull << hp.m) + (U ? (double)(1ull << known) : 0.0));
-  return launch_tiles(M, psi, P.n, view, pass, hp, 1ull << vary, &ba, st, sums, grid_out, other);
+  svp::DevPass at = hp;  // the tile's rows as they lie in the compact state
+  for (int i = 4; i < 7; ++i) at.tq[i] = (uint8_t)std::max(place(P, hp.tq[i]), 4);
+  return launch_tiles(M, psi, basis_state_bits(P), view, pass, at, 1ull << vary, &ba, st, sums, grid_out, other);
+}
+
+int basis_state_bits(const svp::Plan &P) {
+  return std::max(__builtin_popcountll(support(P, (int)P.passes.size() - 1)), 7);
 }
 
 }  // namespace svj

@@ -99,11 +99,11 @@ cudaError_t launch_pass(const Module *M, float2 *psi, int n, const svk::DevPlanV
                         const svp::DevPass &hp, cudaStream_t st, double *sums = nullptr,
                         unsigned *grid_out = nullptr, const float2 *other = nullptr);
 
-// A pass of a plan with Plan::basis: the state starts as |x>.  bytes (may be null): the
-// state bytes the pass reads and writes (the inner variant's last one: reads of `other`).
+// A pass of a plan with Plan::basis (inner variant): the state starts as |x>; psi holds
+// 2^basis_state_bits amplitudes, the support of the passes before the last.
 cudaError_t launch_basis_pass(const Module *M, float2 *psi, const svk::DevPlanView &view, const svp::Plan &P, int pass,
-                              uint64_t x, cudaStream_t st, double *sums, unsigned *grid_out, const float2 *other,
-                              double *bytes);
+                              uint64_t x, cudaStream_t st, double *sums, unsigned *grid_out, const float2 *other);
+int basis_state_bits(const svp::Plan &P);
 
 // Upper bound of the CTAs one pass launch uses (sizes the sums buffer).
 unsigned max_pass_grid();
