@@ -20,11 +20,13 @@ __global__ void branch_sum_kernel(const float2 *__restrict__ A, int nA, const fl
                                   int t, const uint64_t *__restrict__ xa, const uint64_t *__restrict__ xb,
                                   double scale, double *__restrict__ out) {
   const int j = blockIdx.x;
-  const uint64_t a0 = xa[j], b0 = xb[j];
   const uint64_t branches = 1ull << t;
+  // (nA < 0: A holds branch_gather_kernel's slices)
+  const uint64_t a0 = nA < 0 ? (uint64_t)j << t : xa[j], b0 = xb[j];
+  const int sa = nA < 0 ? 0 : nA;
   double sr = 0.0, si = 0.0;
   for (uint64_t l = threadIdx.x; l < branches; l += blockDim.x) {
-    const float2 a = A[a0 + (l << nA)];
+    const float2 a = A[a0 + (l << sa)];
     const float2 b = B[b0 + (l << nB)];
     sr += (double)a.x * b.x - (double)a.y * b.y;
     si += (double)a.x * b.y + (double)a.y * b.x;
@@ -44,6 +46,13 @@ __global__ void branch_sum_kernel(const float2 *__restrict__ A, int nA, const fl
     out[2 * j] = rr[0] * scale;
     out[2 * j + 1] = ri[0] * scale;
   }
+}
+
+// The 2^t branch amplitudes of each bitstring's half index xa[j], one bitstring after the other.
+__global__ void branch_gather_kernel(const float2 *__restrict__ A, int nA, int t, const uint64_t *__restrict__ xa,
+                                     uint64_t count, float2 *__restrict__ out) {
+  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < count; i += (uint64_t)gridDim.x * blockDim.x)
+    out[i] = A[xa[i >> t] + ((i & ((1ull << t) - 1)) << nA)];
 }
 
 // The tensor form of the same sum (§2, Eqs. 6-7: the full state is a sum over branches
@@ -235,6 +244,15 @@ cudaError_t launch_outer_sum(const float2 *A, const float2 *B, const OuterShape 
   if (S.nA < 1 || S.nB < 1 || ta + tb > 30) return cudaErrorInvalidValue;
   const bool scaled = S.signs > 0 || scale.y != 0.f;
   (scaled ? outer_sum_kernel<true> : outer_sum_kernel<false>)<<<1u << (ta + tb), 256, 0, st>>>(A, B, S, scale, ta, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_branch_gather(const float2 *A, int nA, int t, const uint64_t *xa, uint64_t m, float2 *out,
+                                 cudaStream_t st) {
+  const uint64_t count = m << t;
+  if (count == 0) return cudaSuccess;
+  const unsigned grid = (unsigned)std::min<uint64_t>((count + kBlock - 1) / kBlock, (uint64_t)device_sm_count() * 8);
+  branch_gather_kernel<<<grid, kBlock, 0, st>>>(A, nA, t, xa, count, out);
   return cudaGetLastError();
 }
 

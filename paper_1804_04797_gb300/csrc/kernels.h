@@ -55,7 +55,11 @@ cudaError_t launch_gather(const float2 *psi, const uint64_t *bits, int64_t m, do
 cudaError_t launch_gather_prob(const float2 *psi, const uint64_t *bits, int64_t m, double *out,
                                cudaStream_t st);
 
-// K6: out[2j..2j+1] = scale * sum_l A[xa_j + (l << nA)] * B[xb_j + (l << nB)], fp64.
+// out[(j << t) + l] = A[xa_j + (l << nA)] for l < 2^t.
+cudaError_t launch_branch_gather(const float2 *A, int nA, int t, const uint64_t *xa, uint64_t m, float2 *out,
+                                 cudaStream_t st);
+// K6: out[2j..2j+1] = scale * sum_l A[xa_j + (l << nA)] * B[xb_j + (l << nB)], fp64 (nA < 0: A
+// holds what launch_branch_gather wrote).
 cudaError_t launch_branch_sum(const float2 *A, int nA, const float2 *B, int nB, int t, const uint64_t *xa,
                               const uint64_t *xb, int m, double scale, double *out, cudaStream_t st);
 
