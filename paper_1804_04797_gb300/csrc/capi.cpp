@@ -370,6 +370,7 @@ sv_status run_plan(sv_state *s, const svp::Plan &P, const svk::DevPlanView &view
     double *partials = sums && p + 1 == P.passes.size() ? s->d_sums + 2 : nullptr;
     prof_begin(s);
     cudaError_t e = fused ? svk::launch_fused_pass(s->psi, s->n, view, (int)p, hp, s->stream, f16, P.rk)
+                    : jit && p == 0 && P.fork ? svj::launch_fork_pass(jit, s->psi, view, P, s->stream)
                     : jit ? svj::launch_pass(jit, s->psi, s->n, view, (int)p, hp, s->stream, partials, &grid)
                           : svk::launch_tile_pass(s->psi, s->n, static_cast<unsigned char *>(s->d_plan) + s->block_offset[p],
                                                   s->block_bytes[p], hp.m, P.rk, s->stream);
@@ -538,11 +539,20 @@ sv_status autotune_plain(sv_state *s, const std::vector<svp::Gate> &g, const svp
 
 }  // namespace
 
+// The pending fork of a branch tree's prefix, by a kernel of its own.
+static sv_status fork_now(sv_state *s) {
+  const cudaError_t e = svk::launch_fork(s->psi, s->n - s->fork, s->n, s->stream);
+  s->fork = 0;
+  if (e != cudaSuccess) { s->broken = true; return cuda_fail(e, "branch fork"); }
+  return SV_OK;
+}
+
 sv_status apply_gates(sv_state *s, const std::vector<svp::Gate> &g) {
   sv_status st;
   if ((st = set_device(s)) != SV_OK) return st;
   s->sums_valid = false;
   if (s->opts.precision == SV_PREC_PERGATE || s->n < 6) {
+    if (s->fork > 0 && (st = fork_now(s)) != SV_OK) return st;
     // (a tensor-core request on a state this small is a plain fallback too)
     if (s->prof && (s->opts.precision == SV_PREC_TF32X3 || s->opts.precision == SV_PREC_F16X3)) s->plain_fallbacks += 1;
     return apply_pergate(s, g);
@@ -597,6 +607,7 @@ sv_status apply_gates(sv_state *s, const std::vector<svp::Gate> &g) {
         for (svp::DevPass &dp : P.passes) dp.flags |= svp::PF_RAW;
     }
     std::string jerr;
+    if (svj::pass_can_fork(P, s->fork)) P.fork = s->fork;
     jit = svj::get_module(P, po.rk, &jerr);
     if (!jit && s->opts.jit == 1) return fail(SV_ERR_CUDA, jerr.c_str());
     if (!jit && po.fused) {
@@ -626,6 +637,8 @@ sv_status apply_gates(sv_state *s, const std::vector<svp::Gate> &g) {
   if (kfused)
     for (const svp::DevPass &dp : P.passes)
       if (dp.stage_count > 256) return fail(SV_ERR_ARG, "fused path: more than 256 stages in one pass");
+  if (s->fork > 0 && P.fork == 0 && (st = fork_now(s)) != SV_OK) return st;
+  s->fork = 0;
   svk::DevPlanView view;
   if ((st = upload_plan(s, P, &view, !kfused && !jit)) != SV_OK) return st;
   if ((st = run_plan(s, P, view, kfused, f16, jit)) != SV_OK) return st;
@@ -1091,6 +1104,13 @@ sv_status sv_jit_check(int n_qubits, const sv_gate *gates, size_t n_gates, const
                                                       : svj::pass_source(P, po.rk, last, true),
                       "sm_103a", &cubin, &lg2);
     if (!lg2.empty()) lg += "inner last pass: " + lg2;
+    if (ok && svj::pass_can_fork(P, 1)) {
+      // and the first pass as it forks a prefix
+      P.fork = 1;
+      ok = svj::compile(svj::pipe_pass_source(P, po.rk, 0, false), "sm_103a", &cubin, &lg2);
+      if (!lg2.empty()) lg += "forking first pass: " + lg2;
+      P.fork = 0;
+    }
     if (ok && !fresh_state && po.layout == 1) {
       // and every pass as it runs from a basis state
       P.basis = true;

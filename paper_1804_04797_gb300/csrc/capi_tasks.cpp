@@ -174,6 +174,7 @@ sv_status plan_cut(const sv_lattice *lat, const sv_cut *cut, CutPlan *C, bool fu
 sv_status run_branch_tree(sv_state *full, int n_base, const std::vector<svp::Gate> &g) {
   const int n_all = full->n;
   int active = 0;  // branch bits in the prefix
+  int fork = 0;    // the highest of them, not yet in memory: the next segment's first pass forks
   std::vector<svp::Gate> seg;
   bool first = true;
   auto flush = [&]() -> sv_status {
@@ -188,6 +189,8 @@ sv_status run_branch_tree(sv_state *full, int n_base, const std::vector<svp::Gat
     view.one_shape = full->one_shape;
     view.fresh = first;
     view.user_writes = true;
+    view.fork = fork;
+    fork = 0;
     const sv_status st = apply_gates(&view, seg);
     const sv_status werr = st == SV_OK ? take_pending_error(&view) : st;
     if (view.d_plan) cudaFree(view.d_plan);
@@ -208,8 +211,7 @@ sv_status run_branch_tree(sv_state *full, int n_base, const std::vector<svp::Gat
     if (top >= active) {
       sv_status st = flush();
       if (st != SV_OK) return st;
-      const cudaError_t e = svk::launch_fork(full->psi, n_base + active, n_base + top + 1, full->stream);
-      if (e != cudaSuccess) { full->broken = true; return cuda_fail(e, "branch fork"); }
+      fork = top + 1 - active;
       active = top + 1;
     }
     seg.push_back(x);

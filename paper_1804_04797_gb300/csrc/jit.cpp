@@ -461,11 +461,14 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
   for (int i = 0; i < dp.nt; ++i) vary |= ((U >> dp.ntq[i]) & 1ull) << i;
   for (int i = 0; i < m; ++i) masked = masked || !((U >> dp.tq[i]) & 1ull);
   const bool all_tiles = vary == (dp.nt >= 64 ? ~0ull : (1ull << dp.nt) - 1);
+  const bool fork = P.fork > 0 && pass == 0;  // reads the prefix, scaled (Plan::fork)
   // C statements: this CTA's tile of turn `var` (leaves the loop after the last one)
   auto tile_stmt = [&](const char *var) {
-    std::string t = std::string("const unsigned long long tile_") + (all_tiles ? "id" : "j") + " = tile_of<RUN>(" + var +
-                    ", num_tiles);\n      if (tile_" + (all_tiles ? "id" : "j") + " >= num_tiles) break;\n";
-    if (all_tiles) return t;
+    const std::string id = all_tiles && !fork ? "tile_id" : "tile_j";
+    std::string t = "const unsigned long long " + id + " = tile_of<RUN>(" + var + ", num_tiles);\n      if (" + id +
+                    " >= num_tiles) break;\n";
+    if (all_tiles && !fork) return t;
+    if (fork) return t + "      const unsigned long long tile_id = first_tile + tile_j;\n";
     t += "      const unsigned long long tile_id = ba.fixed";
     for (int i = 0, from = 0; i < dp.nt;) {
       if (!((vary >> i) & 1ull)) { ++i; continue; }
@@ -516,7 +519,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
   os << "\nextern \"C\" __global__ void __launch_bounds__(" << NT << ", 1)\nsv_pass"
      << "(float2 *__restrict__ psi, svk::DevPlanView plan, unsigned long long num_tiles, double *sums,\n"
      << "        const float2 *__restrict__ other, const __grid_constant__ TmaDesc tmap"
-     << (P.basis ? ", const svk::BasisArgs ba" : "") << ") {\n"
+     << (P.basis ? ", const svk::BasisArgs ba" : fork ? ", const unsigned long long first_tile" : "") << ") {\n"
      << "  constexpr int G = " << G << ", S = " << S << ", TG = " << TG << ";\n"
      << "  constexpr int RUN = " << (mma ? 0 : tile_run_log()) << ";  // runs of 2^RUN neighbouring tiles per turn\n"
      << "  constexpr unsigned TILE_BYTES = " << (8u << m) << "u;\n"
@@ -584,7 +587,8 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
   } else {
     os << "      if (lane == 0) mbar_arrive_tx(&full_bar[s], TILE_BYTES);\n"
        << "      __syncwarp();\n"
-       << "      const int row0 = (int)((" << tile_base_expr(P, dp) << ") >> 4);\n"
+       << "      const int row0 = (int)(((" << tile_base_expr(P, dp) << ")"
+       << (fork ? " & " + std::to_string((1ull << (P.n - P.fork)) - 1) + "ull" : std::string()) << ") >> 4);\n"
        << "      unsigned char *dst = smem + s * TILE_BYTES;\n"
        << "      for (int j = lane; j < " << nbox << "; j += 32) {\n"
        << "        int row = row0;\n"
@@ -904,6 +908,18 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
              << "        R[p] = f2(x.x, x.z);\n        I[p] = f2(x.y, x.w);\n      }\n      }\n";
         }
       } else os << "      load_group_rx<" << (s == 0 ? "true" : "false") << ">(tile, a0, rx, R, I);\n";
+      if (s == 0 && fork) {  // as fork_kernel scales, operation by operation
+        const svk::ForkScale f = svk::fork_scale(P.fork);
+        char hi[32], lo[32];
+        std::snprintf(hi, sizeof(hi), "%.9ef", f.hi);
+        std::snprintf(lo, sizeof(lo), "%.9ef", f.lo);
+        auto scaled = [&](const std::string &v) {
+          return f.lo == 0.f ? v + " * " + hi : "fmaf(" + v + ", " + hi + ", " + v + " * " + lo + ")";
+        };
+        os << "#pragma unroll\n      for (int p = 0; p < kP; ++p) {\n"
+           << "        R[p] = f2(" << scaled("R[p].x") << ", " << scaled("R[p].y") << ");\n"
+           << "        I[p] = f2(" << scaled("I[p].x") << ", " << scaled("I[p].y") << ");\n      }\n";
+      }
       if (last_stage && direct)  // the slot is free once every thread of the group has read it
         os << "      fence_proxy_async();\n      mbar_arrive(&empty_bar[slot]);\n";
       emit_stage_ops(os, P, st, &pending, true);
@@ -1272,6 +1288,15 @@ bool pass_is_pipelined(const svp::Plan &P, int pass) {
   return P.layout == 1 && P.passes[(size_t)pass].stage_count > 0 && pass_pipe_shape(P, pass, &g, &s);
 }
 
+bool pass_can_fork(const svp::Plan &P, int bits) {
+  if (bits < 1 || P.basis || P.mma || P.passes.empty() || !pass_is_pipelined(P, 0)) return false;
+  const svp::DevPass &hp = P.passes[0];
+  if ((hp.flags & (svp::PF_INIT_UNIFORM | svp::PF_INIT_ZERO)) || P.n - hp.m < bits) return false;
+  for (int i = 0; i < hp.m; ++i)
+    if (hp.tq[i] >= P.n - bits) return false;
+  return true;
+}
+
 std::string any_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) {
   return pass_is_pipelined(P, pass) ? pipe_pass_source(P, kpr, pass, inner) : pass_source(P, kpr, pass, inner);
 }
@@ -1429,9 +1454,10 @@ cudaError_t prepare_passes(const Module *Mc, const svp::Plan &P) {
 
 unsigned max_pass_grid() { return (unsigned)svk::device_sm_count() * 32u; }  // <= 32 CTAs per SM
 
-// One pass over `tiles` tiles; ba: a basis plan's arguments (else null).
+// One pass over `tiles` tiles; more: the last argument of a kernel that takes one (a basis plan's
+// BasisArgs, the first tile of a forking pass), else null.
 static cudaError_t launch_tiles(const Module *Mc, float2 *psi, int n, const svk::DevPlanView &view, int pass,
-                                const svp::DevPass &hp, uint64_t tiles, svk::BasisArgs *ba, cudaStream_t st, double *sums,
+                                const svp::DevPass &hp, uint64_t tiles, void *more, cudaStream_t st, double *sums,
                                 unsigned *grid_out, const float2 *other) {
   Module *M = const_cast<Module *>(Mc);
   const Driver &D = driver();
@@ -1463,7 +1489,7 @@ static cudaError_t launch_tiles(const Module *Mc, float2 *psi, int n, const svk:
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
-    void *args[] = {&psi, &v, &num_tiles, &sums, &other, &map, ba};
+    void *args[] = {&psi, &v, &num_tiles, &sums, &other, &map, more};
     r = D.launch(f, (unsigned)grid, 1, 1, (unsigned)threads, 1, 1, (unsigned)smem, (CUstream)st, args, nullptr);
   } else {
     void *args[] = {&psi, &v, &num_tiles, &sums, &other};
@@ -1476,6 +1502,18 @@ cudaError_t launch_pass(const Module *M, float2 *psi, int n, const svk::DevPlanV
                         const svp::DevPass &hp, cudaStream_t st, double *sums, unsigned *grid_out,
                         const float2 *other) {
   return launch_tiles(M, psi, n, view, pass, hp, 1ull << (n - hp.m), nullptr, st, sums, grid_out, other);
+}
+
+cudaError_t launch_fork_pass(const Module *M, float2 *psi, const svk::DevPlanView &view, const svp::Plan &P,
+                             cudaStream_t st) {
+  const svp::DevPass &hp = P.passes[0];
+  const uint64_t tiles = 1ull << (P.n - hp.m);
+  unsigned long long first = tiles >> P.fork;  // the prefix's own tiles come last
+  cudaError_t e = launch_tiles(M, psi, P.n, view, 0, hp, tiles - first, &first, st, nullptr, nullptr, nullptr);
+  const uint64_t own = first;
+  first = 0;
+  if (e == cudaSuccess) e = launch_tiles(M, psi, P.n, view, 0, hp, own, &first, st, nullptr, nullptr, nullptr);
+  return e;
 }
 
 cudaError_t launch_basis_pass(const Module *M, float2 *psi, const svk::DevPlanView &view, const svp::Plan &P, int pass,

@@ -105,6 +105,13 @@ cudaError_t launch_basis_pass(const Module *M, float2 *psi, const svk::DevPlanVi
                               uint64_t x, cudaStream_t st, double *sums, unsigned *grid_out, const float2 *other);
 int basis_state_bits(const svp::Plan &P);
 
+// Whether a plan's first pass can read a state whose `bits` highest qubits are still |+> from
+// the slice in which they are 0, the only one in memory (Plan::fork): none of them is in its tiles.
+bool pass_can_fork(const svp::Plan &P, int bits);
+// That pass: the tiles of the other slices first, then the slice's own.
+cudaError_t launch_fork_pass(const Module *M, float2 *psi, const svk::DevPlanView &view, const svp::Plan &P,
+                             cudaStream_t st);
+
 // Upper bound of the CTAs one pass launch uses (sizes the sums buffer).
 unsigned max_pass_grid();
 

@@ -227,14 +227,12 @@ cudaError_t launch_fork(float2 *psi, int n_cur, int n_new, cudaStream_t st) {
   if (n_new <= n_cur) return cudaSuccess;
   if (n_cur < 1) return cudaErrorInvalidValue;
   const int k = n_new - n_cur;
-  // f = 2^{-k/2}: exact for even k; for odd k, 1/sqrt2 as the float nearest plus the rest
-  const double f = std::ldexp(1.0, -(k / 2)) * ((k & 1) ? 0.70710678118654752440 : 1.0);
-  const float hi = (float)f, lo = (float)(f - (double)hi);
+  const ForkScale f = fork_scale(k);
   const uint64_t pairs = 1ull << (n_cur - 1);
   uint64_t grid = (pairs + 255) / 256;
   const uint64_t cap = (uint64_t)device_sm_count() * 16;
   if (grid > cap) grid = cap;
-  fork_kernel<<<(unsigned)grid, 256, 0, st>>>(reinterpret_cast<float4 *>(psi), pairs, k, n_cur, hi, lo);
+  fork_kernel<<<(unsigned)grid, 256, 0, st>>>(reinterpret_cast<float4 *>(psi), pairs, k, n_cur, f.hi, f.lo);
   return cudaGetLastError();
 }
 

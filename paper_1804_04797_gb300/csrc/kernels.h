@@ -5,6 +5,8 @@
 
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include "plan.h"
 
 namespace svk {
@@ -67,6 +69,13 @@ int device_sm_count();
 
 // Fork of a branch tree: psi[i + (c << n_cur)] = 2^{-(n_new - n_cur)/2} psi[i] for every
 // slice c of the branch bits n_cur..n_new-1 (they were |+> until now), in place.
+struct ForkScale {
+  float hi, lo;  // 2^{-bits/2}: an odd power as the float nearest and the rest
+};
+inline ForkScale fork_scale(int bits) {
+  const double f = std::ldexp(1.0, -(bits / 2)) * ((bits & 1) ? 0.70710678118654752440 : 1.0);
+  return ForkScale{(float)f, (float)(f - (double)(float)f)};
+}
 cudaError_t launch_fork(float2 *psi, int n_cur, int n_new, cudaStream_t st);
 
 // The product of two batched half-states (Eqs. 6-7): A holds 2^t summed branches (bits nA..)

@@ -28,6 +28,9 @@ struct sv_state {
   // kernel keep one shape, so that an amplitude does not change, to the last bit, with the
   // tuning of the state path's shapes (interp_shape)
   bool one_shape = false;
+  // > 0: a branch tree's prefix whose `fork` highest qubits the next plan takes as |+> (memory
+  // holds the slice in which they are 0)
+  int fork = 0;
   // device scratch: packed plan, gather/reduction buffers
   void *d_plan = nullptr;
   size_t d_plan_cap = 0;
