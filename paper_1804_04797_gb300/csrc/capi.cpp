@@ -371,6 +371,9 @@ sv_status run_plan(sv_state *s, const svp::Plan &P, const svk::DevPlanView &view
     prof_begin(s);
     cudaError_t e = fused ? svk::launch_fused_pass(s->psi, s->n, view, (int)p, hp, s->stream, f16, P.rk)
                     : jit && p == 0 && P.fork ? svj::launch_fork_pass(jit, s->psi, view, P, s->stream)
+                    : jit && P.listed && p + 1 == P.passes.size()
+                        ? svj::launch_listed_pass(jit, s->psi, view, P, static_cast<const uint64_t *>(s->d_scratch),
+                                                  s->listed, s->stream)
                     : jit ? svj::launch_pass(jit, s->psi, s->n, view, (int)p, hp, s->stream, partials, &grid)
                           : svk::launch_tile_pass(s->psi, s->n, static_cast<unsigned char *>(s->d_plan) + s->block_offset[p],
                                                   s->block_bytes[p], hp.m, P.rk, s->stream);
@@ -597,6 +600,7 @@ sv_status apply_gates(sv_state *s, const std::vector<svp::Gate> &g) {
   // a tensor-core request on a state (or tile) below 12 qubits runs the plain kernel
   s->plan_fallback = (s->opts.precision == SV_PREC_TF32X3 || s->opts.precision == SV_PREC_F16X3) && !po.fused;
   const svj::Module *jit = nullptr;
+  std::vector<uint64_t> tiles;  // of a listed last pass
   const bool f16 = s->opts.precision == SV_PREC_F16X3;
   if (want_jit) {
     if (po.fused) {  // matrix stages of the plan kernels: their B operands (and the
@@ -608,6 +612,10 @@ sv_status apply_gates(sv_state *s, const std::vector<svp::Gate> &g) {
     }
     std::string jerr;
     if (svj::pass_can_fork(P, s->fork)) P.fork = s->fork;
+    if (s->needed && svj::last_pass_tiles(P, *s->needed, s->all_of, &tiles)) {
+      P.listed = true;
+      P.all_of = s->all_of;
+    }
     jit = svj::get_module(P, po.rk, &jerr);
     if (!jit && s->opts.jit == 1) return fail(SV_ERR_CUDA, jerr.c_str());
     if (!jit && po.fused) {
@@ -641,6 +649,13 @@ sv_status apply_gates(sv_state *s, const std::vector<svp::Gate> &g) {
   s->fork = 0;
   svk::DevPlanView view;
   if ((st = upload_plan(s, P, &view, !kfused && !jit)) != SV_OK) return st;
+  if (P.listed) {
+    if ((st = ensure_device_buffer(&s->d_scratch, &s->d_scratch_cap, tiles.size() * sizeof(uint64_t))) != SV_OK) return st;
+    const cudaError_t e = cudaMemcpyAsync(s->d_scratch, tiles.data(), tiles.size() * sizeof(uint64_t),
+                                          cudaMemcpyHostToDevice, s->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "tile list upload");
+    s->listed = tiles.size();
+  }
   if ((st = run_plan(s, P, view, kfused, f16, jit)) != SV_OK) return st;
   s->fresh = false;
   if (kfused && (st = check_fused_error(s, view)) != SV_OK) return st;
@@ -1110,6 +1125,14 @@ sv_status sv_jit_check(int n_qubits, const sv_gate *gates, size_t n_gates, const
       ok = svj::compile(svj::pipe_pass_source(P, po.rk, 0, false), "sm_103a", &cubin, &lg2);
       if (!lg2.empty()) lg += "forking first pass: " + lg2;
       P.fork = 0;
+    }
+    if (ok && svj::pass_is_pipelined(P, last)) {
+      // and the last pass on listed tiles, two qubits outside them taking every value
+      P.listed = true;
+      for (int i = 0; i < P.passes.back().nt && i < 4; i += 3) P.all_of |= 1ull << P.passes.back().ntq[i];
+      ok = svj::compile(svj::pipe_pass_source(P, po.rk, last, false), "sm_103a", &cubin, &lg2);
+      if (!lg2.empty()) lg += "listed last pass: " + lg2;
+      P.listed = false;
     }
     if (ok && !fresh_state && po.layout == 1) {
       // and every pass as it runs from a basis state

@@ -171,13 +171,16 @@ sv_status plan_cut(const sv_lattice *lat, const sv_cut *cut, CutPlan *C, bool fu
 // prefix is forked (replicated into the new slices, times 2^{-1/2} per new bit).  The
 // result is the state the whole list would give on all n_base + t qubits; the work before
 // each fork is done once instead of once per branch.
-sv_status run_branch_tree(sv_state *full, int n_base, const std::vector<svp::Gate> &g) {
+// needed (may be null): the indices that will be read of it, at every value of the first tf
+// branch bits.
+sv_status run_branch_tree(sv_state *full, int n_base, const std::vector<svp::Gate> &g,
+                          const std::vector<uint64_t> *needed = nullptr, int tf = 0) {
   const int n_all = full->n;
   int active = 0;  // branch bits in the prefix
   int fork = 0;    // the highest of them, not yet in memory: the next segment's first pass forks
   std::vector<svp::Gate> seg;
   bool first = true;
-  auto flush = [&]() -> sv_status {
+  auto flush = [&](bool last) -> sv_status {
     if (seg.empty() && !first) return SV_OK;
     sv_state view;  // the prefix: n_base + active qubits of the same buffer
     view.n = n_base + active;
@@ -191,6 +194,10 @@ sv_status run_branch_tree(sv_state *full, int n_base, const std::vector<svp::Gat
     view.user_writes = true;
     view.fork = fork;
     fork = 0;
+    if (last && needed) {
+      view.needed = needed;
+      view.all_of = ((1ull << tf) - 1) << n_base;
+    }
     const sv_status st = apply_gates(&view, seg);
     const sv_status werr = st == SV_OK ? take_pending_error(&view) : st;
     if (view.d_plan) cudaFree(view.d_plan);
@@ -209,14 +216,14 @@ sv_status run_branch_tree(sv_state *full, int n_base, const std::vector<svp::Gat
     if (x.q0 >= n_base) top = x.q0 - n_base;
     if (svp::kind_two_qubit(x.kind) && x.q1 >= n_base) top = std::max(top, x.q1 - n_base);
     if (top >= active) {
-      sv_status st = flush();
+      sv_status st = flush(false);
       if (st != SV_OK) return st;
       fork = top + 1 - active;
       active = top + 1;
     }
     seg.push_back(x);
   }
-  sv_status st = flush();
+  sv_status st = flush(true);
   if (st != SV_OK) return st;
   if (active < n_all - n_base) {  // branch bits no gate touches: still |+>
     const cudaError_t e = svk::launch_fork(full->psi, n_base + active, n_all, full->stream);
@@ -261,7 +268,7 @@ extern "C" sv_status sv_branch_amplitudes(const sv_lattice *lat, const sv_cut *c
   std::memset(&o, 0, sizeof(o));
   if (opts) o = *opts;
   // bitstring -> half indices, with the implicit branch bits fixed by the output bits
-  std::vector<uint64_t> xab(2 * m);
+  std::vector<uint64_t> xs_a(m), xs_b(m);
   std::vector<double> sign(m, 1.0);
   for (size_t k = 0; k < m; ++k) {
     uint64_t xa = 0, xb = 0;
@@ -274,8 +281,8 @@ extern "C" sv_status sv_branch_amplitudes(const sv_lattice *lat, const sv_cut *c
     for (const auto &f : C.fix_b) xb |= ((bits[k] >> f.second) & 1ull) << (nb + f.first);
     for (const auto &sg : C.signs)
       if (((bits[k] >> sg.first) & 1ull) && ((bits[k] >> sg.second) & 1ull)) sign[k] = -sign[k];
-    xab[k] = xa;
-    xab[m + k] = xb;
+    xs_a[k] = xa;
+    xs_b[k] = xb;
   }
   // Half B takes half A's place: of A the sum needs 2^tf amplitudes a bitstring, which are put
   // aside first.  Two halves side by side have to be allocated and freed, 0.85 us a MB (42
@@ -295,7 +302,7 @@ extern "C" sv_status sv_branch_amplitudes(const sv_lattice *lat, const sv_cut *c
     return st;
   }
   A.s->one_shape = B.s->one_shape = true;
-  if ((st = run_branch_tree(A.s, na, C.ga)) != SV_OK) return st;
+  if ((st = run_branch_tree(A.s, na, C.ga, &xs_a, C.tf)) != SV_OK) return st;
   sv_state *s = A.s;
   auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t o_out = align(2 * m * sizeof(uint64_t)), o_a = o_out + align(2 * m * sizeof(double));
@@ -305,10 +312,12 @@ extern "C" sv_status sv_branch_amplitudes(const sv_lattice *lat, const sv_cut *c
   uint64_t *d_x = reinterpret_cast<uint64_t *>(d);
   double *d_out = reinterpret_cast<double *>(d + o_out);
   float2 *d_a = reinterpret_cast<float2 *>(d + o_a);
+  std::vector<uint64_t> xab(xs_a);
+  xab.insert(xab.end(), xs_b.begin(), xs_b.end());
   cudaError_t e = m == 0 ? cudaSuccess : cudaMemcpyAsync(d_x, xab.data(), 2 * m * sizeof(uint64_t), cudaMemcpyHostToDevice, s->stream);
   if (e == cudaSuccess && share) e = svk::launch_branch_gather(s->psi, na, C.tf, d_x, m, d_a, s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "sv_branch_amplitudes");
-  if ((st = run_branch_tree(B.s, nb, C.gb)) != SV_OK) return st;
+  if ((st = run_branch_tree(B.s, nb, C.gb, &xs_b, C.tf)) != SV_OK) return st;
   if (m == 0) return SV_OK;
   // each slice carries 2^{-t_half/2}: the sum is rescaled by 2^{(ta + tb)/2}
   const double scale = std::pow(2.0, 0.5 * (C.ta + C.tb));

@@ -251,6 +251,14 @@ uint64_t placed(const svp::Plan &P, uint64_t index) {
   return v;
 }
 
+// The tile index bits of the last pass at which the qubits of Plan::all_of lie.
+uint64_t listed_bits(const svp::Plan &P) {
+  const svp::DevPass &dp = P.passes.back();
+  uint64_t v = 0;
+  for (int i = 0; i < dp.nt; ++i) v |= ((P.all_of >> dp.ntq[i]) & 1ull) << i;
+  return v;
+}
+
 // C expression of a stage's group addressing for thread index `var`: the XOR over its
 // group-index bits of the stage's per-bit offsets (L: shared-memory byte offset, 32-bit;
 // G: global index offset, 64-bit; `whole`: in the whole state, where P's is kept compactly), as
@@ -462,18 +470,24 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
   for (int i = 0; i < m; ++i) masked = masked || !((U >> dp.tq[i]) & 1ull);
   const bool all_tiles = vary == (dp.nt >= 64 ? ~0ull : (1ull << dp.nt) - 1);
   const bool fork = P.fork > 0 && pass == 0;  // reads the prefix, scaled (Plan::fork)
+  // the listed tiles alone (Plan::listed)
+  const bool listed = last && P.listed;
   // C statements: this CTA's tile of turn `var` (leaves the loop after the last one)
   auto tile_stmt = [&](const char *var) {
-    const std::string id = all_tiles && !fork ? "tile_id" : "tile_j";
+    const std::string id = all_tiles && !fork && !listed ? "tile_id" : "tile_j";
     std::string t = "const unsigned long long " + id + " = tile_of<RUN>(" + var + ", num_tiles);\n      if (" + id +
                     " >= num_tiles) break;\n";
-    if (all_tiles && !fork) return t;
+    if (id == "tile_id") return t;
     if (fork) return t + "      const unsigned long long tile_id = first_tile + tile_j;\n";
-    t += "      const unsigned long long tile_id = ba.fixed";
+    uint64_t bits = vary;  // the tile index bits that tile_j runs through
+    if (listed) bits = listed_bits(P);
+    t += listed ? "      const unsigned long long tile_id = __ldg(tile_list + (tile_j >> " +
+                      std::to_string(__builtin_popcountll(bits)) + "))"
+                : std::string("      const unsigned long long tile_id = ba.fixed");
     for (int i = 0, from = 0; i < dp.nt;) {
-      if (!((vary >> i) & 1ull)) { ++i; continue; }
+      if (!((bits >> i) & 1ull)) { ++i; continue; }
       int k = i;
-      while (k < dp.nt && ((vary >> k) & 1ull)) ++k;
+      while (k < dp.nt && ((bits >> k) & 1ull)) ++k;
       t += " | (((tile_j >> " + std::to_string(from) + ") & " + std::to_string((1ull << (k - i)) - 1) + "ull) << " +
            std::to_string(i) + ")";
       from += k - i;
@@ -519,7 +533,8 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
   os << "\nextern \"C\" __global__ void __launch_bounds__(" << NT << ", 1)\nsv_pass"
      << "(float2 *__restrict__ psi, svk::DevPlanView plan, unsigned long long num_tiles, double *sums,\n"
      << "        const float2 *__restrict__ other, const __grid_constant__ TmaDesc tmap"
-     << (P.basis ? ", const svk::BasisArgs ba" : fork ? ", const unsigned long long first_tile" : "") << ") {\n"
+     << (P.basis ? ", const svk::BasisArgs ba" : fork ? ", const unsigned long long first_tile"
+         : listed ? ", const unsigned long long *__restrict__ tile_list" : "") << ") {\n"
      << "  constexpr int G = " << G << ", S = " << S << ", TG = " << TG << ";\n"
      << "  constexpr int RUN = " << (mma ? 0 : tile_run_log()) << ";  // runs of 2^RUN neighbouring tiles per turn\n"
      << "  constexpr unsigned TILE_BYTES = " << (8u << m) << "u;\n"
@@ -1502,6 +1517,31 @@ cudaError_t launch_pass(const Module *M, float2 *psi, int n, const svk::DevPlanV
                         const svp::DevPass &hp, cudaStream_t st, double *sums, unsigned *grid_out,
                         const float2 *other) {
   return launch_tiles(M, psi, n, view, pass, hp, 1ull << (n - hp.m), nullptr, st, sums, grid_out, other);
+}
+
+bool last_pass_tiles(const svp::Plan &P, const std::vector<uint64_t> &needed, uint64_t all_of,
+                     std::vector<uint64_t> *tiles) {
+  const int last = (int)P.passes.size() - 1;
+  if (last < 0 || P.basis || P.mma || (last == 0 && P.fork) || !pass_is_pipelined(P, last)) return false;
+  const svp::DevPass &dp = P.passes.back();
+  int all = 0;
+  for (int i = 0; i < dp.nt; ++i) all += (int)((all_of >> dp.ntq[i]) & 1ull);
+  tiles->clear();
+  for (uint64_t x : needed) {
+    uint64_t t = 0;
+    for (int i = 0; i < dp.nt; ++i)
+      if (!((all_of >> dp.ntq[i]) & 1ull)) t |= ((x >> dp.ntq[i]) & 1ull) << i;
+    tiles->push_back(t);
+  }
+  std::sort(tiles->begin(), tiles->end());
+  tiles->erase(std::unique(tiles->begin(), tiles->end()), tiles->end());
+  return !tiles->empty() && (tiles->size() << all) <= (1ull << dp.nt) / 2;
+}
+
+cudaError_t launch_listed_pass(const Module *M, float2 *psi, const svk::DevPlanView &view, const svp::Plan &P,
+                               const uint64_t *tiles, size_t count, cudaStream_t st) {
+  return launch_tiles(M, psi, P.n, view, (int)P.passes.size() - 1, P.passes.back(),
+                      (uint64_t)count << __builtin_popcountll(listed_bits(P)), &tiles, st, nullptr, nullptr, nullptr);
 }
 
 cudaError_t launch_fork_pass(const Module *M, float2 *psi, const svk::DevPlanView &view, const svp::Plan &P,

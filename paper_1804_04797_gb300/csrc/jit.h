@@ -112,6 +112,15 @@ bool pass_can_fork(const svp::Plan &P, int bits);
 cudaError_t launch_fork_pass(const Module *M, float2 *psi, const svk::DevPlanView &view, const svp::Plan &P,
                              cudaStream_t st);
 
+// The tiles of a plan's last pass that hold the needed amplitudes -- every index that agrees with
+// one of `needed` outside the qubits all_of -- as the tile indices with all_of's bits 0.  False
+// where the pass cannot run on them alone or they are more than half of its tiles.
+bool last_pass_tiles(const svp::Plan &P, const std::vector<uint64_t> &needed, uint64_t all_of,
+                     std::vector<uint64_t> *tiles);
+// The last pass (Plan::listed, all_of) on those tiles (a device copy of the list).
+cudaError_t launch_listed_pass(const Module *M, float2 *psi, const svk::DevPlanView &view, const svp::Plan &P,
+                               const uint64_t *tiles, size_t count, cudaStream_t st);
+
 // Upper bound of the CTAs one pass launch uses (sizes the sums buffer).
 unsigned max_pass_grid();
 

@@ -86,6 +86,13 @@ struct Plan {
   // GB300, with a fork kernel and a pass over what it wrote -> so: 3.43 -> 3.15, 6.5 -> 5.89,
   // 3.51 -> 3.47 ms a call.
   int fork = 0;
+  // plan kernels of a state of which few amplitudes are wanted: the last pass runs on listed
+  // tiles, each entry standing for the tiles at every value of the qubits all_of
+  // (launch_listed_pass).  Measured, 42 qubits, 64 bitstrings, three circuits on one GB300, whole
+  // last passes -> listed ones: 3.15 -> 2.87, 5.9 -> 5.13, 3.47 -> 3.02 ms a call; a list of more
+  // than half the tiles is not worth a kernel of its own.
+  bool listed = false;
+  uint64_t all_of = 0;
 };
 
 // Build the plan.  fresh_state: the state is |0..0> and was never written, so a

@@ -31,6 +31,11 @@ struct sv_state {
   // > 0: a branch tree's prefix whose `fork` highest qubits the next plan takes as |+> (memory
   // holds the slice in which they are 0)
   int fork = 0;
+  // not null: of the next plan's result, the amplitudes at these indices, at every value of the
+  // qubits all_of, are all that will be read
+  const std::vector<uint64_t> *needed = nullptr;
+  uint64_t all_of = 0;
+  size_t listed = 0;  // entries of the tile list (in d_scratch) of a plan's listed last pass
   // device scratch: packed plan, gather/reduction buffers
   void *d_plan = nullptr;
   size_t d_plan_cap = 0;
