@@ -343,7 +343,7 @@ sv_status upload_plan(sv_state *s, const svp::Plan &P, svk::DevPlanView *view, b
   view->stages = reinterpret_cast<const svp::DevStage *>(d + o_stage);
   view->ops = reinterpret_cast<const svp::DevOp *>(d + o_op);
   view->mats = reinterpret_cast<const float *>(d + o_mat);
-  view->err = reinterpret_cast<int *>(d + o_err);
+  view->err = s->d_err ? s->d_err : reinterpret_cast<int *>(d + o_err);
   view->gtab = reinterpret_cast<const svp::DevGroupEntry *>(d + o_gt);
   return SV_OK;
 }
@@ -884,6 +884,7 @@ sv_status sv_destroy(sv_state *s) {
   if (s->d_plan) cudaFree(s->d_plan);
   if (s->d_scratch) cudaFree(s->d_scratch);
   if (s->d_sums) cudaFree(s->d_sums);
+  if (s->d_err) cudaFree(s->d_err);
   for (cudaEvent_t ev : s->events) cudaEventDestroy(ev);
   delete s;
   return SV_OK;

@@ -55,6 +55,7 @@ struct sv_state {
   // error word of the last plan run on kernels with bounded waits (the pipelined plan
   // kernels), read by the next call that synchronises the stream; null when none is due
   int *err_pending = nullptr;
+  int *d_err = nullptr;  // not null: the error word of all its plans (else each has its own)
   // the last plan run on this handle (a circuit applied again reuses it and its device
   // copy: no planning, kernel-source hashing or upload)
   bool plan_valid = false;
