@@ -76,10 +76,7 @@ batch_kernel(float2 *__restrict__ states, const unsigned char *__restrict__ bloc
     __syncthreads();
     if (s_stop) break;
     const uint32_t end = min(it.tile + (1u << cp.run), cp.tiles);
-    for (uint32_t t = it.tile; t < end; ++t) {
-      if (t != it.tile) __syncthreads();  // the tile before has been read
-      process_tile<kBatchSlots>(states + cp.state_off, blk, src, tile, t);
-    }
+    for (uint32_t t = it.tile; t < end; ++t) process_tile<kBatchSlots>(states + cp.state_off, blk, src, tile, t);
     __threadfence();  // each thread's stores visible device-wide before the count
     __syncthreads();
     if (tid == 0) atomicAdd(&done[it.cp], end - it.tile);
