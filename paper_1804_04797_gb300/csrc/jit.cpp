@@ -366,35 +366,28 @@ size_t pass_mma_smem(const svp::Plan &P, int pass) {
   return pass_matrix_stages(P, pass) > 0 ? (size_t)2 * 2 * 64 * 64 * (P.mma == 1 ? 2 : 4) : 0;
 }
 
-// Tile streams per compute group of a tensor-core pass (F16x3 2, TF32x3 1; SV_MMA_SHAPE
-// "G,X,S" overrides groups, streams and slots for tuning: TMEM G X columns, S a multiple of
-// G X, shared memory and threads within their limits).
+// SV_MMA_SHAPE "G,S" overrides the compute groups and slots of a tensor-core pass (tuning: within
+// TMEM, shared memory and threads, S a multiple of G).
 namespace {
 struct MmaShape {
-  int g = 0, x = 0, s = 0;
+  int g = 0, s = 0;
 };
 MmaShape mma_shape_env(int mma) {
   static MmaShape env[3];
   static std::once_flag once;
   std::call_once(once, [] {
     const char *e = std::getenv("SV_MMA_SHAPE");
-    int g = 0, x = 0, s = 0;
-    if (e && std::sscanf(e, "%d,%d,%d", &g, &x, &s) == 3 && g >= 1 && x >= 1 && x <= 2 && s % (g * x) == 0)
+    int g = 0, s = 0;
+    if (e && std::sscanf(e, "%d,%d", &g, &s) == 2 && g >= 1 && s >= g && s % g == 0)
       for (int k = 1; k <= 2; ++k) {
         const int cols = k == 1 ? 128 : 256;
         const size_t smem = (size_t)s * 32768 + 2 * 2 * 64 * 64 * (k == 1 ? 2 : 4) + 1024;
-        if (g * x * cols <= 512 && smem <= 227 * 1024 && g * 128 + 96 <= 1024) env[k] = MmaShape{g, x, s};
+        if (g * cols <= 512 && smem <= 216 * 1024 && g * 128 + 96 <= 1024) env[k] = MmaShape{g, s};
       }
   });
   return env[mma];
 }
 }  // namespace
-
-int pass_streams(const svp::Plan &P, int pass) {
-  if (pass_matrix_stages(P, pass) == 0) return 1;
-  const MmaShape e = mma_shape_env(P.mma);
-  return e.g ? e.x : (P.mma == 1 ? 2 : 1);
-}
 
 bool pass_pipe_shape(const svp::Plan &P, int pass, int *groups, int *slots) {
   const int m = P.passes[(size_t)pass].m;
@@ -405,12 +398,16 @@ bool pass_pipe_shape(const svp::Plan &P, int pass, int *groups, int *slots) {
       *slots = e.s;
       return true;
     }
-    // tensor-core passes (12-qubit tiles): two groups of four warps (168 registers a
-    // thread: 11 warps with the producer, storer and MMA warps), each with two tiles in
-    // flight (F16x3: 4 x 128 TMEM columns of A hi, A lo and D) or one (TF32x3: 2 x 256);
-    // shared memory: four 32 KB slots and two B buffers (2 x 16 KB or 2 x 32 KB)
+    // tensor-core passes (12-qubit tiles): groups of four warps, each with a tile in flight.
+    // TF32x3 two (2 x 256 TMEM columns of A hi, A lo and D); F16x3 (128 columns) four where the
+    // CTAs have several tiles each -- a group's instructions wait for one another, so more warps
+    // fill the issue slots although 96 registers spill a little -- and two below that (us at 2 / 4
+    // groups, one GB300: 12 qubits 13.9 / 15.7, 16 32.7 / 33.2, 19 36.3 / 37.3, 20 43.0 / 45.0,
+    // 21 63.8 / 59.8, 22 102 / 88; two tiles in flight for each of two groups, as it was: 14.3,
+    // 32.0, 35.9, 47.8, 62.0, 93.4; 25 qubits 728 -> 696, 28 3.38 -> 3.25 ms, 32 71.4 -> 67.3).
+    // Shared memory: four 32 KB slots and two B buffers (2 x 16 KB or 2 x 32 KB).
     if (m != 12) return false;
-    *groups = 2;
+    *groups = P.mma == 1 && P.n >= 21 ? 4 : 2;
     *slots = 4;
     return true;
   }
@@ -507,13 +504,10 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
   // tensor-core matrix stages (fused packed plans): an MMA warp after the other roles
   const int nms = pass_matrix_stages(P, pass);
   const bool mma = nms > 0;
-  if (mma && (kpr != 4 || TG != 128 || inner || S % (G * pass_streams(P, pass)) != 0))
+  if (mma && (kpr != 4 || TG != 128 || inner || S % G != 0))
     return std::string("#error \"matrix stages need 12-qubit tiles and four register slots\"\n");
   const bool f16 = P.mma == 1;
   const bool restore = mma && (dp.flags & svp::PF_UNITARY) && !(dp.flags & svp::PF_RAW);
-  // tiles a compute group keeps in flight (streams): F16x3 two, alternating at every
-  // matrix stage so that one tile's products run while the group works on the other
-  const int X = pass_streams(P, pass), NSTR = G * X;
   const int MT0 = G * TG + 32 + (direct ? 0 : 32);  // first thread of the MMA warp
   auto row_of = [&](int q) { return place(P, q) < 4 ? 0u : 1u << (place(P, q) - 4); };
   std::string boxrow;  // C statements: row += the row offset of box j
@@ -554,18 +548,17 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
      << "  const int tid = threadIdx.x;\n";
   if (mma) {
     os << "  constexpr int NMS = " << nms << ";                // matrix stages of the pass\n"
-       << "  constexpr int X = " << X << ", NSTR = " << NSTR << ";  // tile streams: X per group, stream g X + x\n"
        << "  constexpr unsigned BSTAGE = " << 2 * 64 * 64 * (f16 ? 2 : 4) << "u;  // one stage's B (hi + lo)\n"
        << "  constexpr uint32_t ACOLS = " << (f16 ? 32 : 64) << "u, CG = " << (f16 ? 128 : 256)
-       << "u;  // TMEM columns: one A part; one stream (A hi, A lo, D)\n"
+       << "u;  // TMEM columns: one A part; one group (A hi, A lo, D)\n"
        << "  constexpr int MT0 = " << MT0 << ";  // the MMA warp\n"
        << "  unsigned char *bring = smem + S * TILE_BYTES;  // two B buffers\n"
-       << "  // a_full[s]: stream s's A is in TMEM; d_full[s]: its products are done; b_full /\n"
+       << "  // a_full[g]: group g's A is in TMEM; d_full[g]: its products are done; b_full /\n"
        << "  // b_free: a B buffer has landed / its products have read it\n"
-       << "  __shared__ __align__(8) unsigned long long a_full[NSTR], d_full[NSTR], b_full[2], b_free[2], drain_bar;\n"
+       << "  __shared__ __align__(8) unsigned long long a_full[G], d_full[G], b_full[2], b_free[2], drain_bar;\n"
        << "  __shared__ uint32_t tmem_base;\n";
     if (restore || f16)
-      os << "  __shared__ float2 nrm[2][NSTR][2][4];  // per tile parity and stream: warp sums of the norm in / out\n";
+      os << "  __shared__ float2 nrm[2][G][2][4];  // per tile parity and group: warp sums of the norm in / out\n";
   }
   os << "  if (tid == 0) {\n"
      << "    P = plan.passes[" << pass << "];\n"
@@ -575,7 +568,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
   else os << "      mbar_init(&empty_bar[s], 1);\n      mbar_init(&done_bar[s], TG);\n";
   os << "    }\n";
   if (mma)
-    os << "    for (int g = 0; g < NSTR; ++g) { mbar_init(&a_full[g], TG); mbar_init(&d_full[g], 1); }\n"
+    os << "    for (int g = 0; g < G; ++g) { mbar_init(&a_full[g], TG); mbar_init(&d_full[g], 1); }\n"
        << "    for (int b = 0; b < 2; ++b) { mbar_init(&b_full[b], 1); mbar_init(&b_free[b], 1); }\n"
        << "    mbar_init(&drain_bar, 1);\n";
   os << "    mbar_init_fence();\n"
@@ -631,12 +624,12 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
        << "      mbar_wait(&full_bar[k % S], (uint32_t)((k / S) & 1), kWaitNs);\n";
   if (mma) {
     os << "  } else if (tid >= MT0) {\n"
-       << "    // MMA warp: for each round of NSTR tiles (stream g's tile j NSTR + g), each matrix\n"
-       << "    // stage s and each stream g, wait for the stream's A and issue its products with\n"
-       << "    // stage s's B; B is streamed from the plan into two buffers one stage ahead.\n"
+       << "    // MMA warp: for each round of G tiles (group g's tile j G + g), each matrix stage s\n"
+       << "    // and each group g, wait for the group's A and issue its products with stage s's B;\n"
+       << "    // B is streamed from the plan into two buffers one stage ahead.\n"
        << "    if (elect_lane()) {\n"
        << "      const unsigned long long mine = tiles_of_cta<RUN>(num_tiles);\n"
-       << "      const unsigned long long rounds = (mine + NSTR - 1) / NSTR, steps = rounds * NMS;\n"
+       << "      const unsigned long long rounds = (mine + G - 1) / G, steps = rounds * NMS;\n"
        << "      const unsigned char *bsrc = reinterpret_cast<const unsigned char *>(plan.mats);\n"
        << "      uint32_t apar = 0;\n"
        << "      bool ok = true;\n"
@@ -652,11 +645,8 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
        << "          if (!mbar_wait(&b_full[buf], (uint32_t)((q >> 1) & 1), kWaitNs)) { ok = false; break; }\n"
        << "          ++landed;\n"
        << "          const uint32_t bh = smem_u32(bring + buf * BSTAGE), bl = bh + BSTAGE / 2;\n"
-       << "          // streams in the order they get ready: every group's first stream, then\n"
-       << "          // every group's second (a group alternates between its streams)\n"
-       << "          for (int gg = 0; gg < NSTR; ++gg) {\n"
-       << "            const int g = (gg % G) * X + gg / G;\n"
-       << "            if (j * NSTR + g >= mine) continue;\n"
+       << "          for (int g = 0; g < G; ++g) {\n"
+       << "            if (j * G + g >= mine) continue;\n"
        << "            if (!mbar_wait(&a_full[g], (apar >> g) & 1u, kWaitNs)) { ok = false; break; }\n"
        << "            apar ^= 1u << g;\n"
        << "            fence_after();\n"
@@ -667,7 +657,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
        << "            // step before this one have left it: behind this step's first products\n"
        << "            // (at the step's end its latency was exposed: 28 qubits F16x3 8.11 -> 7.93 ms,\n"
        << "            // 25 qubits TF32x3 1.14 -> 1.10 ms)\n"
-       << "            if (gg == 0 && q + 1 < steps) {\n"
+       << "            if (g == 0 && q + 1 < steps) {\n"
        << "              if (q >= 1 && !mbar_wait(&b_free[buf ^ 1], (uint32_t)(((q - 1) >> 1) & 1), kWaitNs)) { ok = false; break; }\n"
        << "              mbar_arrive_tx(&b_full[buf ^ 1], BSTAGE);\n"
        << "              bulk_g2s(bring + (buf ^ 1) * BSTAGE, bsrc + b_src((s + 1) % NMS), BSTAGE, &b_full[buf ^ 1]);\n"
@@ -714,20 +704,22 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
     // ---- compute groups with tensor-core matrix stages (streams alternate per stage;
     // the stream is a run-time index, so each stage's code exists once)
     os << "  } else {\n"
-       << "    // group g runs streams X g + x (x < X); stream s takes the CTA's tiles s, s + NSTR, ...,\n"
-       << "    // tile i in slot i mod S (S a multiple of NSTR: each slot serves one stream).  The streams\n"
-       << "    // alternate at every stage: one stream's products run while the group works on the other.\n"
+       << "    // group g takes tiles g, g + G, ...: tile i in slot i mod S (S a multiple of G).  One\n"
+       << "    // group's products run while the others work.\n"
        << "    const int g = tid / TG, t = tid % TG;\n"
        << "    const int bar_id = 1 + g;\n"
        << "    const uint32_t tl = tmem + ((uint32_t)(32 * ((tid >> 5) & 3)) << 16);  // this thread's TMEM lane\n"
        << "    Regs R, I;\n"
-       << "    for (unsigned long long i = (unsigned long long)(X * g), k = 0;; i += NSTR, ++k) {\n"
-       << "      if (tile_of<RUN>(i, num_tiles) >= num_tiles) break;\n"
-       << "      // streams of the group with a tile in this round\n"
-       << "      const int nx = (X == 2 && tile_of<RUN>(i + 1, num_tiles) < num_tiles) ? 2 : 1;\n"
-       << "      float sc0 = 1.f, sc1 = 1.f;  // F16: the tile's scale (power of two) from its first product\n"
-       << "      bool okm0 = true, okm1 = true;    // every product wait of the tile succeeded\n"
-       << "      bool stop = false;\n";
+       << "    const uint32_t tg = tl + (uint32_t)g * CG;\n"
+       << "    for (unsigned long long i = (unsigned long long)g, k = 0;; i += G, ++k) {\n"
+       << "      const unsigned long long tile_id = tile_of<RUN>(i, num_tiles);\n"
+       << "      if (tile_id >= num_tiles) break;\n"
+       << "      const int slot = (int)(i % S);\n"
+       << "      float4 *tile = reinterpret_cast<float4 *>(smem + slot * TILE_BYTES);\n"
+       << "      const uint32_t W = ((uint32_t)tile_id << " << (m - 1 - kpr) << ") | (uint32_t)t;\n"
+       << "      float sc = 1.f;   // F16: the tile's scale (power of two) from its first product\n"
+       << "      bool okm = true;  // every product wait of the tile succeeded\n"
+       << "      (void)W; (void)sc;\n";
     const int ns = dp.stage_count;
     // matrix-stage index of each stage (-1: no products), and the first one
     std::vector<int> msi(ns, -1);
@@ -738,26 +730,6 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
         if (first_ms < 0) first_ms = s;
       }
     int pending = 0;  // factors 1/2 pending (lowered square roots only; none in these plans)
-    // the loop over the streams of a round, with the stream's tile in scope
-    auto stream_loop_head = [&]() {
-      os << "#pragma unroll 1\n"
-         << "      for (int x = 0; x < nx; ++x) {\n"
-         << "        const unsigned long long ii = i + (unsigned long long)x;\n"
-         << "        const unsigned long long tile_id = tile_of<RUN>(ii, num_tiles);\n"
-         << "        const int slot = (int)(ii % S);\n"
-         << "        float4 *tile = reinterpret_cast<float4 *>(smem + slot * TILE_BYTES);\n"
-         << "        const int sx = X * g + x;  // the stream\n"
-         << "        const uint32_t tgx = tl + (uint32_t)sx * CG;\n"
-         << "        const uint32_t W = ((uint32_t)tile_id << " << (m - 1 - kpr) << ") | (uint32_t)t;\n"
-         << "        float scx = x ? sc1 : sc0;\n"
-         << "        bool okm = x ? okm1 : okm0;\n"
-         << "        (void)tile; (void)tgx; (void)W; (void)scx; (void)okm;\n";
-    };
-    auto stream_loop_tail = [&]() {
-      os << "        if (x) { sc1 = scx; okm1 = okm; } else { sc0 = scx; okm0 = okm; }\n"
-         << "      }\n"
-         << "      if (stop) break;\n";
-    };
     auto stage_head = [&](uint32_t si) {
       os << "        const uint32_t rx[" << kpr << "] = {";
       for (int j = 0; j < kpr; ++j)
@@ -791,14 +763,14 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
         // reference, and (F16x3) the tile's scale
         os << "        {\n"
            << "          const float2 w = warp_sum2(row_norm2(R, I));\n"
-           << "          if (lane == 0) nrm[k & 1][sx][0][t >> 5] = w;\n";
+           << "          if (lane == 0) nrm[k & 1][g][0][t >> 5] = w;\n";
         if (f16)
           os << "          group_sync(bar_id, TG);\n"
-             << "          scx = tile_scale(nrm[k & 1][sx][0]);\n";
+             << "          sc = tile_scale(nrm[k & 1][g][0]);\n";
         os << "        }\n";
       }
       os << "        matrix_pre<" << (f16 ? "true" : "false") << ", " << (f16 && first ? "true" : "false")
-         << ">(R, I, scx, tgx, tgx + ACOLS, &a_full[sx]);\n"
+         << ">(R, I, sc, tg, tg + ACOLS, &a_full[g]);\n"
          << "        }\n";
     };
     // second half (or a whole stage without products): D back, the ops, the store
@@ -811,13 +783,13 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
       os << "        int ph = 0;\n        bool zero = false;\n";
       if (msi[s] >= 0)
         os << "        okm &= matrix_post<" << (f16 ? "true" : "false")
-           << ">(R, I, tgx + 2 * ACOLS, &d_full[sx], (uint32_t)((k * NMS + " << msi[s] << ") & 1));\n";
+           << ">(R, I, tg + 2 * ACOLS, &d_full[g], (uint32_t)((k * NMS + " << msi[s] << ") & 1));\n";
       else
         emit_load(s);
       emit_stage_ops(os, P, st, &pending);
       emit_stage_end(os, &pending, last_stage);
       if (last_stage && f16)  // back from the tile's scale (exact)
-        os << "        scale_all(R, I, inv_pow2(scx));\n";
+        os << "        scale_all(R, I, inv_pow2(sc));\n";
       if (last_stage && restore) {
         // every gate of a PF_UNITARY pass acts inside the tile, so the tile keeps its
         // norm: the products' truncating fp32 accumulation (~0.3 ulp of every output per
@@ -825,9 +797,9 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
         // rounded
         os << "        {  // the tile's norm restored\n"
            << "          const float2 w = warp_sum2(row_norm2(R, I));\n"
-           << "          if (lane == 0) nrm[k & 1][sx][1][t >> 5] = w;\n"
+           << "          if (lane == 0) nrm[k & 1][g][1][t >> 5] = w;\n"
            << "          group_sync(bar_id, TG);\n"
-           << "          const float delta = restore_delta(nrm[k & 1][sx][0], nrm[k & 1][sx][1]);\n"
+           << "          const float delta = restore_delta(nrm[k & 1][g][0], nrm[k & 1][g][1]);\n"
            << "          const uint32_t seed = (uint32_t)tile_id * 0x85EBCA6Bu + (uint32_t)(tile_id >> 32) * 0xC2B2AE35u +\n"
            << "                                " << (uint32_t)pass * 0x27D4EB2Fu << "u + (uint32_t)t * 0x165667B1u;\n"
            << "          scale_row_sr(R, I, delta, seed);\n"
@@ -835,7 +807,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
       }
       if (!last_stage) {
         os << "        store_group_rx(tile, a0, rx, R, I);\n"
-           << "        if (group_any(bar_id, TG, !okm)) { if (t == 0) atomicExch(plan.err, 5); stop = true; break; }\n"
+           << "        if (group_any(bar_id, TG, !okm)) { if (t == 0) atomicExch(plan.err, 5); break; }\n"
            << "        }\n";
         return;
       }
@@ -866,20 +838,12 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
          << "          *reinterpret_cast<float4 *>(psi + gb + go[p]) = make_float4(R[p].x, I[p].x, R[p].y, I[p].y);\n"
          << "        }\n";
     };
-    // the schedule: each stream's tile and A of stage 0, then per stage each stream's D
-    // and the next stage's A
-    stream_loop_head();
-    os << "        {\n"
-       << "          const bool ok = mbar_wait(&full_bar[slot], (uint32_t)((ii / S) & 1), kWaitNs);\n"
-       << "          if (group_any(bar_id, TG, !ok)) { if (t == 0) atomicExch(plan.err, 3); stop = true; break; }\n"
-       << "        }\n";
+    os << "      const bool ok = mbar_wait(&full_bar[slot], (uint32_t)((i / S) & 1), kWaitNs);\n"
+       << "      if (group_any(bar_id, TG, !ok)) { if (t == 0) atomicExch(plan.err, 3); break; }\n";
     emit_pre(0);
-    stream_loop_tail();
     for (int s = 0; s < ns; ++s) {
-      stream_loop_head();
       emit_post(s);
       emit_pre(s + 1);
-      stream_loop_tail();
     }
     os << "    }\n  }\n";
   } else {
