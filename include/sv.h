@@ -265,7 +265,7 @@ sv_status sv_branch_counts(const sv_lattice *lat, const sv_cut *cut, int counts[
 
 /* Simulate count independent lattice circuits (each with its own state, 6..28 qubits;
  * §2's circuits at many sizes) in ONE persistent launch over a work queue of (circuit,
- * pass, tile) items: all circuits' first passes, then all second passes, ...  An item
+ * pass, run of tiles) items: all circuits' first passes, then all second passes, ...  An item
  * waits for its circuit's previous pass with a bounded spin; if a wait gives up the call
  * returns SV_ERR_TIMEOUT (no hang).  The launch, the queue reset and the per-circuit fp64
  * statistics are captured once in a CUDA graph and replayed while the same lattice list
@@ -351,8 +351,9 @@ sv_status sv_inner_product(sv_state *a, sv_state *b, double *out_re_im);
  * |psi> = U1 H^n |0> is computed once, and for every bitstring x, |phi_x> = U2^dagger |x>
  * and alpha_x = <phi_x|psi>; on plan-specialised kernels (sv_options.jit) the last pass
  * of phi_x sums <phi_x|psi> instead of storing phi_x, and the passes before it run only
- * where phi_x can differ from zero.  Two n-qubit states are allocated
- * (2 x 8 x 2^n bytes, at most n = 34 on GB300) and freed on return; out_re_im receives
+ * where phi_x can differ from zero and need no memory beside that.  |psi> and, where
+ * phi_x is stored, a second n-qubit state are allocated (8 x 2^n bytes each, at most n = 34 on
+ * GB300) and freed on return; out_re_im receives
  * 2m doubles.  A split_layer at or beyond the depth gives the plain amplitudes of the
  * full state. */
 sv_status sv_amplitudes_by_inner_product(const sv_lattice *lat, int split_layer, const uint64_t *bits, size_t m,

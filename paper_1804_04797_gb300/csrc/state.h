@@ -110,10 +110,10 @@ sv_status apply_gates_inner(sv_state *s, const std::vector<svp::Gate> &g, const 
 // kernels that keep to the amplitudes which can differ from zero: outside the tile qubits of
 // its passes so far the state is still x, so the first passes touch 2^12, 2^20, ... of its 2^n
 // amplitudes, nothing is cleared beforehand, and the last pass reads little besides `with`
-// (28 qubits, 8 layers back, 3 passes, one GB300: 0.16 ms a
-// bitstring, 2.4 ms with the state cleared and whole passes).  Those amplitudes alone have
-// memory, in index order (there the call went from 5.6 to 4.6 ms when the backward state's
-// 2 GB were no longer allocated and freed).  *done = false where these kernels are not in use for with's options or NVRTC is
+// (28 qubits, 8 layers back, 3 passes, one GB300: 0.16 ms a bitstring, 2.4 ms with the state
+// cleared and whole passes).  Those amplitudes alone have memory, in index order (there the
+// call went from 5.6 to 4.6 ms when the backward state's 2 GB were no longer allocated and
+// freed).  *done = false where these kernels are not in use for with's options or NVRTC is
 // missing.
 sv_status basis_inner_products(sv_state *with, const std::vector<svp::Gate> &g, const uint64_t *xs, size_t m,
                                double *out, bool *done);
