@@ -611,8 +611,12 @@ sv_status apply_gates(sv_state *s, const std::vector<svp::Gate> &g) {
         for (svp::DevPass &dp : P.passes) dp.flags |= svp::PF_RAW;
     }
     std::string jerr;
-    if (svj::pass_can_fork(P, s->fork)) P.fork = s->fork;
-    if (s->needed && svj::last_pass_tiles(P, *s->needed, s->all_of, &tiles)) {
+    // a fork read by its pass and a listed last pass pay from the size at which the device, not
+    // the queueing, sets the pace (cut amplitudes with F16x3 halves: 42 qubits, halves of 26..28
+    // with their branches, 3.80 -> 3.19 and 7.28 -> 5.66 ms; 36 qubits, halves of 22, 1.24 -> 1.28)
+    const bool large = s->n >= kJitMinQubits || s->opts.jit == 1;
+    if (large && svj::pass_can_fork(P, s->fork)) P.fork = s->fork;
+    if (large && s->needed && svj::last_pass_tiles(P, *s->needed, s->all_of, &tiles)) {
       P.listed = true;
       P.all_of = s->all_of;
     }
@@ -1111,15 +1115,17 @@ sv_status sv_jit_check(int n_qubits, const sv_gate *gates, size_t n_gates, const
   std::vector<std::string> cubins;
   std::string lg;
   bool ok = svj::compile_plan(P, po.rk, "sm_103a", &cubins, &lg, "");
-  if (ok && !P.passes.empty() && !tc) {
-    // and the last pass as the inner-product variant (the backward states of the
-    // inner-product amplitudes)
+  if (ok && !P.passes.empty()) {
     std::string cubin, lg2;
     const int last = (int)P.passes.size() - 1;
-    ok = svj::compile(svj::pass_is_pipelined(P, last) ? svj::pipe_pass_source(P, po.rk, last, true)
-                                                      : svj::pass_source(P, po.rk, last, true),
-                      "sm_103a", &cubin, &lg2);
-    if (!lg2.empty()) lg += "inner last pass: " + lg2;
+    if (!tc) {
+      // and the last pass as the inner-product variant (the backward states of the
+      // inner-product amplitudes)
+      ok = svj::compile(svj::pass_is_pipelined(P, last) ? svj::pipe_pass_source(P, po.rk, last, true)
+                                                        : svj::pass_source(P, po.rk, last, true),
+                        "sm_103a", &cubin, &lg2);
+      if (!lg2.empty()) lg += "inner last pass: " + lg2;
+    }
     if (ok && svj::pass_can_fork(P, 1)) {
       // and the first pass as it forks a prefix
       P.fork = 1;
@@ -1135,7 +1141,7 @@ sv_status sv_jit_check(int n_qubits, const sv_gate *gates, size_t n_gates, const
       if (!lg2.empty()) lg += "listed last pass: " + lg2;
       P.listed = false;
     }
-    if (ok && !fresh_state && po.layout == 1) {
+    if (ok && !tc && !fresh_state && po.layout == 1) {
       // and every pass as it runs from a basis state
       P.basis = true;
       for (size_t p = 0; ok && p < P.passes.size(); ++p) {

@@ -474,10 +474,10 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
   const bool fork = P.fork > 0 && pass == 0;  // reads the prefix, scaled (Plan::fork)
   // the listed tiles alone (Plan::listed)
   const bool listed = last && P.listed;
-  // C statements: this CTA's tile of turn `var` (leaves the loop after the last one)
-  auto tile_stmt = [&](const char *var) {
+  // C statements: this CTA's tile of turn i (leaves the loop after the last one)
+  const std::string this_tile = [&]() {
     const std::string id = all_tiles && !fork && !listed ? "tile_id" : "tile_j";
-    std::string t = "const unsigned long long " + id + " = tile_of<RUN>(" + var + ", num_tiles);\n      if (" + id +
+    std::string t = "const unsigned long long " + id + " = tile_of<RUN>(i, num_tiles);\n      if (" + id +
                     " >= num_tiles) break;\n";
     if (id == "tile_id") return t;
     if (fork) return t + "      const unsigned long long tile_id = first_tile + tile_j;\n";
@@ -496,7 +496,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
       i = k;
     }
     return t + ";\n      (void)tile_id;\n";
-  };
+  }();
   // the last stage's output: straight from registers (whole rows per quarter warp), or
   // back into the slot in memory order, written out by a storer warp with TMA stores
   const bool direct = inner || pipe_direct_store(P, pass);
@@ -514,6 +514,19 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
   for (int b = 0; b + 7 < m; ++b)
     boxrow += "        if ((j >> " + std::to_string(b) + ") & 1) row += " + std::to_string(row_of(dp.tq[7 + b])) + ";\n";
   std::ostringstream os;
+  // the fork's scaling of a loaded group, as fork_kernel does it, operation by operation
+  auto emit_fork_scale = [&]() {
+    const svk::ForkScale f = svk::fork_scale(P.fork);
+    char hi[32], lo[32];
+    std::snprintf(hi, sizeof(hi), "%.9ef", f.hi);
+    std::snprintf(lo, sizeof(lo), "%.9ef", f.lo);
+    auto scaled = [&](const std::string &v) {
+      return f.lo == 0.f ? v + " * " + hi : "fmaf(" + v + ", " + hi + ", " + v + " * " + lo + ")";
+    };
+    os << "#pragma unroll\n      for (int p = 0; p < kP; ++p) {\n"
+       << "        R[p] = f2(" << scaled("R[p].x") << ", " << scaled("R[p].y") << ");\n"
+       << "        I[p] = f2(" << scaled("I[p].x") << ", " << scaled("I[p].y") << ");\n      }\n";
+  };
   os << "// pipelined tile-pass kernel of one pass of a plan\n#define SV_PACK_R " << kpr
      << "\n#include \"tile_pack.cuh\"\n#include \"tile_pipe.cuh\"\n"
      << (mma ? "#include \"tile_mma.cuh\"\n" : "")
@@ -597,7 +610,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
      << "    // producer warp: tile i of this CTA into slot i mod S once the slot is empty\n"
      << "    unsigned long long i = 0;\n"
      << "    for (;; ++i) {\n"
-     << "      " << tile_stmt("i")
+     << "      " << this_tile
      << "      const int s = (int)(i % S);\n"
      << "      bool ok = i < S || mbar_wait(&empty_bar[s], (uint32_t)((i / S - 1) & 1), kWaitNs);\n"
      << "      ok = __all_sync(0xffffffffu, ok);\n"
@@ -681,7 +694,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
        << "    // storer warp: tile i out of its slot once its group has written it back, then\n"
        << "    // the slot goes to the producer\n"
        << "    for (unsigned long long i = 0;; ++i) {\n"
-       << "      " << tile_stmt("i")
+       << "      " << this_tile
        << "      const int s = (int)(i % S);\n"
        << "      bool ok = mbar_wait(&done_bar[s], (uint32_t)((i / S) & 1), kWaitNs);\n"
        << "      ok = __all_sync(0xffffffffu, ok);\n"
@@ -712,8 +725,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
        << "    Regs R, I;\n"
        << "    const uint32_t tg = tl + (uint32_t)g * CG;\n"
        << "    for (unsigned long long i = (unsigned long long)g, k = 0;; i += G, ++k) {\n"
-       << "      const unsigned long long tile_id = tile_of<RUN>(i, num_tiles);\n"
-       << "      if (tile_id >= num_tiles) break;\n"
+       << "      " << this_tile
        << "      const int slot = (int)(i % S);\n"
        << "      float4 *tile = reinterpret_cast<float4 *>(smem + slot * TILE_BYTES);\n"
        << "      const uint32_t W = ((uint32_t)tile_id << " << (m - 1 - kpr) << ") | (uint32_t)t;\n"
@@ -747,6 +759,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
     auto emit_load = [&](int s) {
       if (s == 0 && init) os << "        init_regs(R, I, P, W);\n";
       else os << "        load_group_rx<" << (s == 0 ? "true" : "false") << ">(tile, a0, rx, R, I);\n";
+      if (s == 0 && fork) emit_fork_scale();
       if (s + 1 == ns && direct)  // the slot is free once every thread of the group has read it
         os << "        fence_proxy_async();\n        mbar_arrive(&empty_bar[slot]);\n";
     };
@@ -853,7 +866,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
        << "    const int g = tid / TG, t = tid % TG;\n"
        << "    const int bar_id = 1 + g;\n"
        << "    for (unsigned long long i = g;; i += G) {\n"
-       << "      " << tile_stmt("i")
+       << "      " << this_tile
        << "      const int slot = (int)(i % S);\n"
        << "      const bool ok = mbar_wait(&full_bar[slot], (uint32_t)((i / S) & 1), kWaitNs);\n"
        << "      if (group_any(bar_id, TG, !ok)) { if (t == 0) atomicExch(plan.err, 3); break; }\n"
@@ -905,18 +918,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
              << "        R[p] = f2(x.x, x.z);\n        I[p] = f2(x.y, x.w);\n      }\n      }\n";
         }
       } else os << "      load_group_rx<" << (s == 0 ? "true" : "false") << ">(tile, a0, rx, R, I);\n";
-      if (s == 0 && fork) {  // as fork_kernel scales, operation by operation
-        const svk::ForkScale f = svk::fork_scale(P.fork);
-        char hi[32], lo[32];
-        std::snprintf(hi, sizeof(hi), "%.9ef", f.hi);
-        std::snprintf(lo, sizeof(lo), "%.9ef", f.lo);
-        auto scaled = [&](const std::string &v) {
-          return f.lo == 0.f ? v + " * " + hi : "fmaf(" + v + ", " + hi + ", " + v + " * " + lo + ")";
-        };
-        os << "#pragma unroll\n      for (int p = 0; p < kP; ++p) {\n"
-           << "        R[p] = f2(" << scaled("R[p].x") << ", " << scaled("R[p].y") << ");\n"
-           << "        I[p] = f2(" << scaled("I[p].x") << ", " << scaled("I[p].y") << ");\n      }\n";
-      }
+      if (s == 0 && fork) emit_fork_scale();
       if (last_stage && direct)  // the slot is free once every thread of the group has read it
         os << "      fence_proxy_async();\n      mbar_arrive(&empty_bar[slot]);\n";
       emit_stage_ops(os, P, st, &pending, true);
@@ -1286,7 +1288,7 @@ bool pass_is_pipelined(const svp::Plan &P, int pass) {
 }
 
 bool pass_can_fork(const svp::Plan &P, int bits) {
-  if (bits < 1 || P.basis || P.mma || P.passes.empty() || !pass_is_pipelined(P, 0)) return false;
+  if (bits < 1 || P.basis || P.passes.empty() || !pass_is_pipelined(P, 0)) return false;
   const svp::DevPass &hp = P.passes[0];
   if ((hp.flags & (svp::PF_INIT_UNIFORM | svp::PF_INIT_ZERO)) || P.n - hp.m < bits) return false;
   for (int i = 0; i < hp.m; ++i)
@@ -1504,7 +1506,7 @@ cudaError_t launch_pass(const Module *M, float2 *psi, int n, const svk::DevPlanV
 bool last_pass_tiles(const svp::Plan &P, const std::vector<uint64_t> &needed, uint64_t all_of,
                      std::vector<uint64_t> *tiles) {
   const int last = (int)P.passes.size() - 1;
-  if (last < 0 || P.basis || P.mma || (last == 0 && P.fork) || !pass_is_pipelined(P, last)) return false;
+  if (last < 0 || P.basis || (last == 0 && P.fork) || !pass_is_pipelined(P, last)) return false;
   const svp::DevPass &dp = P.passes.back();
   int all = 0;
   for (int i = 0; i < dp.nt; ++i) all += (int)((all_of >> dp.ntq[i]) & 1ull);
