@@ -714,8 +714,7 @@ std::string pipe_pass_source(const svp::Plan &P, int kpr, int pass, bool inner) 
        << "    bulk_wait_all();  // the stores have completed before the CTA exits\n";
   }
   if (mma) {
-    // ---- compute groups with tensor-core matrix stages (streams alternate per stage;
-    // the stream is a run-time index, so each stage's code exists once)
+    // ---- compute groups with tensor-core matrix stages
     os << "  } else {\n"
        << "    // group g takes tiles g, g + G, ...: tile i in slot i mod S (S a multiple of G).  One\n"
        << "    // group's products run while the others work.\n"
