@@ -13,7 +13,7 @@ namespace svk {
 // `first` is its first item.
 struct BatchCP {
   uint64_t state_off;  // float2 offset of the circuit's state in the batch buffer
-  uint32_t block;        // offset of the pass's block (interp_dev.h) in the batch program
+  uint64_t block;      // offset of the pass's block (interp_dev.h) in the batch program
   uint32_t block_bytes;
   uint32_t prev;       // BatchCP index of the circuit's previous pass (kNoPrev if first)
   uint32_t tiles;      // tiles of this pass

@@ -201,9 +201,11 @@ bool lower_interp(const Plan &P, InterpProgram *out) {
     h.gate_count = (uint32_t)L.gates.size();
     const size_t o_stage = sizeof(IHead), o_step = o_stage + stages.size() * sizeof(IStage);
     const size_t o_gate = o_step + L.steps.size() * sizeof(IStep);
-    h.bytes = (uint32_t)(o_gate + L.gates.size() * sizeof(IGate));
+    const size_t bytes = o_gate + L.gates.size() * sizeof(IGate);
+    if (bytes > 0xffffffffull) return false;
+    h.bytes = (uint32_t)bytes;
     const size_t at = out->blocks.size();
-    out->offset.push_back((uint32_t)at);
+    out->offset.push_back(at);
     out->bytes.push_back(h.bytes);
     out->blocks.resize(at + h.bytes);
     std::memcpy(&out->blocks[at], &h, sizeof(h));

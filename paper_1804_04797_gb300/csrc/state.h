@@ -65,7 +65,8 @@ struct sv_state {
   const svj::Module *plan_jit = nullptr;
   svk::DevPlanView plan_view{};
   // a plan on the interpreting kernel: where each pass's block lies in d_plan
-  std::vector<uint32_t> block_offset, block_bytes;
+  std::vector<uint64_t> block_offset;
+  std::vector<uint32_t> block_bytes;
   // the norm sums (sum p, sum p^2) of the current state, computed by the last pass of a
   // plan-kernel run as it wrote the state: d_sums[0..1]; d_sums[2..] per-CTA partials.
   // Any other write of the state clears sums_valid; a state the caller can write
