@@ -46,6 +46,28 @@ sv_status ensure_device_buffer(void **buf, size_t *cap, size_t need) {
   return SV_OK;
 }
 
+sv_status upload(sv_state *s, void *dst, std::vector<char> &&bytes, const char *what) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s->stream, &capture) != cudaSuccess) cudaGetLastError();
+  const bool keep = s->keep_uploads || capture == cudaStreamCaptureStatusActive;
+  sv_state::Upload &u = s->uploads[s->upload_at % 4];
+  cudaError_t e = cudaSuccess;
+  if (keep) {
+    s->kept_uploads.push_back(std::move(bytes));
+  } else {  // the source of the fourth copy before this one makes way, once that copy is done
+    ++s->upload_at;
+    e = u.copied ? cudaEventSynchronize(u.copied) : cudaEventCreateWithFlags(&u.copied, cudaEventDisableTiming);
+    if (e != cudaSuccess) return cuda_fail(e, what);
+    u.bytes = std::move(bytes);
+  }
+  const std::vector<char> &src = keep ? s->kept_uploads.back() : u.bytes;
+  e = cudaMemcpyAsync(dst, src.data(), src.size(), cudaMemcpyHostToDevice, s->stream);
+  if (e == cudaSuccess && !keep) e = cudaEventRecord(u.copied, s->stream);
+  if (e != cudaSuccess) return cuda_fail(e, what);
+  if (s->prof) s->h2d += (double)src.size();
+  return SV_OK;
+}
+
 svp::Options plan_options(const sv_options &o) {
   svp::Options p;
   // the interpreting and tensor-core kernels take up to 13-qubit tiles; 14 only with
@@ -309,10 +331,7 @@ sv_status upload_plan(sv_state *s, const svp::Plan &P, svk::DevPlanView *view, b
     if (!svp::lower_interp(P, &prog)) return fail(SV_ERR_ARG, "the plan has no interpreter form");
     sv_status st = ensure_device_buffer(&s->d_plan, &s->d_plan_cap, prog.blocks.size());
     if (st != SV_OK) return st;
-    s->h_plan.assign(prog.blocks.begin(), prog.blocks.end());
-    cudaError_t e = cudaMemcpyAsync(s->d_plan, s->h_plan.data(), s->h_plan.size(), cudaMemcpyHostToDevice, s->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "plan upload");
-    if (s->prof) s->h2d += (double)s->h_plan.size();
+    if ((st = upload(s, s->d_plan, bytes_of(prog.blocks), "plan upload")) != SV_OK) return st;
     s->block_offset = prog.offset;
     s->block_bytes = prog.bytes;
     *view = svk::DevPlanView{};
@@ -328,16 +347,13 @@ sv_status upload_plan(sv_state *s, const svp::Plan &P, svk::DevPlanView *view, b
   const size_t total = o_err + 256;
   sv_status st = ensure_device_buffer(&s->d_plan, &s->d_plan_cap, total);
   if (st != SV_OK) return st;
-  s->h_plan.assign(total, 0);
-  if (!P.passes.empty()) std::memcpy(&s->h_plan[o_pass], P.passes.data(), P.passes.size() * sizeof(svp::DevPass));
-  if (!P.stages.empty()) std::memcpy(&s->h_plan[o_stage], P.stages.data(), P.stages.size() * sizeof(svp::DevStage));
-  if (!P.ops.empty()) std::memcpy(&s->h_plan[o_op], P.ops.data(), P.ops.size() * sizeof(svp::DevOp));
-  if (!P.mats.empty()) std::memcpy(&s->h_plan[o_mat], P.mats.data(), P.mats.size() * sizeof(float));
-  if (!P.gtab.empty())
-    std::memcpy(&s->h_plan[o_gt], P.gtab.data(), P.gtab.size() * sizeof(svp::DevGroupEntry));
-  cudaError_t e = cudaMemcpyAsync(s->d_plan, s->h_plan.data(), total, cudaMemcpyHostToDevice, s->stream);
-  if (e != cudaSuccess) return cuda_fail(e, "plan upload");
-  if (s->prof) s->h2d += (double)total;
+  std::vector<char> host(total, 0);
+  if (!P.passes.empty()) std::memcpy(&host[o_pass], P.passes.data(), P.passes.size() * sizeof(svp::DevPass));
+  if (!P.stages.empty()) std::memcpy(&host[o_stage], P.stages.data(), P.stages.size() * sizeof(svp::DevStage));
+  if (!P.ops.empty()) std::memcpy(&host[o_op], P.ops.data(), P.ops.size() * sizeof(svp::DevOp));
+  if (!P.mats.empty()) std::memcpy(&host[o_mat], P.mats.data(), P.mats.size() * sizeof(float));
+  if (!P.gtab.empty()) std::memcpy(&host[o_gt], P.gtab.data(), P.gtab.size() * sizeof(svp::DevGroupEntry));
+  if ((st = upload(s, s->d_plan, std::move(host), "plan upload")) != SV_OK) return st;
   char *d = static_cast<char *>(s->d_plan);
   view->passes = reinterpret_cast<const svp::DevPass *>(d + o_pass);
   view->stages = reinterpret_cast<const svp::DevStage *>(d + o_stage);
@@ -655,9 +671,7 @@ sv_status apply_gates(sv_state *s, const std::vector<svp::Gate> &g) {
   if ((st = upload_plan(s, P, &view, !kfused && !jit)) != SV_OK) return st;
   if (P.listed) {
     if ((st = ensure_device_buffer(&s->d_scratch, &s->d_scratch_cap, tiles.size() * sizeof(uint64_t))) != SV_OK) return st;
-    const cudaError_t e = cudaMemcpyAsync(s->d_scratch, tiles.data(), tiles.size() * sizeof(uint64_t),
-                                          cudaMemcpyHostToDevice, s->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "tile list upload");
+    if ((st = upload(s, s->d_scratch, bytes_of(tiles), "tile list upload")) != SV_OK) return st;
     s->listed = tiles.size();
   }
   if ((st = run_plan(s, P, view, kfused, f16, jit)) != SV_OK) return st;
@@ -890,6 +904,8 @@ sv_status sv_destroy(sv_state *s) {
   if (s->d_sums) cudaFree(s->d_sums);
   if (s->d_err) cudaFree(s->d_err);
   for (cudaEvent_t ev : s->events) cudaEventDestroy(ev);
+  for (sv_state::Upload &u : s->uploads)
+    if (u.copied) cudaEventDestroy(u.copied);
   delete s;
   return SV_OK;
 }

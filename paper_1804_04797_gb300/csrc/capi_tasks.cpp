@@ -184,6 +184,7 @@ sv_status run_branch_tree(sv_state *full, int n_base, const std::vector<svp::Gat
   std::vector<svp::Gate> seg;
   bool first = true;
   full->user_writes = true;  // (no norm sums)
+  full->keep_uploads = true;
   if (!full->d_err) {
     cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&full->d_err), sizeof(int));
     if (e == cudaSuccess) e = cudaMemsetAsync(full->d_err, 0, sizeof(int), full->stream);
@@ -315,8 +316,9 @@ extern "C" sv_status sv_branch_amplitudes(const sv_lattice *lat, const sv_cut *c
   float2 *d_a = reinterpret_cast<float2 *>(d + o_a);
   std::vector<uint64_t> xab(xs_a);
   xab.insert(xab.end(), xs_b.begin(), xs_b.end());
-  cudaError_t e = m == 0 ? cudaSuccess : cudaMemcpyAsync(d_x, xab.data(), 2 * m * sizeof(uint64_t), cudaMemcpyHostToDevice, s->stream);
-  if (e == cudaSuccess && share) e = svk::launch_branch_gather(s->psi, na, C.tf, d_x, m, d_a, s->stream);
+  if (m && (st = upload(s, d_x, bytes_of(xab), "sv_branch_amplitudes")) != SV_OK) return st;
+  cudaError_t e = cudaSuccess;
+  if (share) e = svk::launch_branch_gather(s->psi, na, C.tf, d_x, m, d_a, s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "sv_branch_amplitudes");
   if ((st = run_branch_tree(B.s, nb, C.gb, &xs_b, C.tf)) != SV_OK) return st;
   if (m == 0) return finish();

@@ -16,6 +16,12 @@ struct Module;
 }
 
 struct sv_state {
+  // The source of a copy to the device that may still be queued: pageable memory, which the copy
+  // may read as late as it runs on the stream.
+  struct Upload {
+    std::vector<char> bytes;
+    cudaEvent_t copied = nullptr;  // not null: recorded behind the copy
+  };
   int n = 0;
   float2 *psi = nullptr;  // 2^n complex64 amplitudes on the device
   bool owns = false;      // allocated by sv_create (freed by sv_destroy)
@@ -39,9 +45,15 @@ struct sv_state {
   // device scratch: packed plan, gather/reduction buffers
   void *d_plan = nullptr;
   size_t d_plan_cap = 0;
-  std::vector<char> h_plan;
   void *d_scratch = nullptr;
   size_t d_scratch_cap = 0;
+  // sources of the last copies, taken in turn (upload), and those kept until the handle goes:
+  // all of them with keep_uploads (a call's own handle, destroyed once its work is done), and
+  // those of copies recorded in a graph
+  Upload uploads[4];
+  unsigned upload_at = 0;
+  bool keep_uploads = false;
+  std::vector<std::vector<char>> kept_uploads;
   // profiling: event pairs around each pass launch
   bool prof = false;
   std::vector<cudaEvent_t> events;
@@ -89,6 +101,13 @@ constexpr int kJitMinQubits = 24;
 
 sv_status cuda_fail(cudaError_t e, const char *what);
 sv_status ensure_device_buffer(void **buf, size_t *cap, size_t need);
+// Copy host bytes to dst on the handle's stream; they stay as they are until the copy has read them.
+sv_status upload(sv_state *s, void *dst, std::vector<char> &&bytes, const char *what);
+template <class T>
+std::vector<char> bytes_of(const std::vector<T> &v) {
+  const char *p = reinterpret_cast<const char *>(v.data());
+  return std::vector<char>(p, p + v.size() * sizeof(T));
+}
 svp::Options plan_options(const sv_options &o);
 // The plan options sv_apply_circuit uses for an n-qubit state; *want_jit: the plain path
 // is to run on plan-specialised kernels.

@@ -1,0 +1,19 @@
+"""What the host code may rely on while the device lags behind it (tests/fake_device.cpp)."""
+import pytest
+
+import host_cpp
+from paper_1804_04797_gb300 import sv
+
+SOURCES = ['capi.cpp', 'capi_tasks.cpp', 'capi_batch.cpp', 'plan.cpp', 'interp.cpp', 'generator.cpp']
+
+
+@pytest.fixture(scope='module')
+def fake_device(tmp_path_factory):
+    return host_cpp.build(tmp_path_factory.mktemp('fake_device'), 'fake_device', SOURCES)
+
+
+@pytest.mark.parametrize('jit,precision', [(-1, sv.SV_PREC_PLAIN), (1, sv.SV_PREC_PLAIN), (0, sv.SV_PREC_F16X3)])
+def test_sources_of_queued_copies_stay_as_they_are(fake_device, jit, precision):
+    # (memory that is given back is overwritten at once)
+    r = host_cpp.run(fake_device, 'uploads', jit, precision, env={'MALLOC_PERTURB_': '165'})
+    assert r.returncode == 0, r.stdout + r.stderr
