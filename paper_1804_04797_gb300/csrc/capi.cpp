@@ -739,12 +739,12 @@ sv_status basis_inner_products(sv_state *with, const std::vector<svp::Gate> &g, 
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "inner product pass");
   s->err_pending = view.err;
-  if ((st = take_pending_error(s)) != SV_OK) return st;
+  if ((st = take_pending_error(s)) != SV_OK || (st = take_pending_error(with)) != SV_OK) return st;
   *done = true;
   return SV_OK;
 }
 
-sv_status apply_gates_inner(sv_state *s, const std::vector<svp::Gate> &g, const sv_state *with, double *out,
+sv_status apply_gates_inner(sv_state *s, const std::vector<svp::Gate> &g, sv_state *with, double *out,
                             bool *fused) {
   *fused = false;
   sv_status st;
@@ -811,7 +811,8 @@ sv_status apply_gates_inner(sv_state *s, const std::vector<svp::Gate> &g, const 
   }
   for (size_t p = 0; p < P.passes.size(); ++p)
     if (svj::pass_is_pipelined(P, (int)p)) s->err_pending = s->plan_view.err;
-  const sv_status werr = take_pending_error(s);
+  sv_status werr = take_pending_error(s);
+  if (werr == SV_OK) werr = take_pending_error(with);
   // the last pass did not store: the state is not the circuit's result
   s->broken = true;
   if (werr != SV_OK) return werr;

@@ -374,6 +374,7 @@ extern "C" sv_status sv_inner_product(sv_state *a, sv_state *b, double *out_re_i
   if (e == cudaSuccess) e = cudaMemcpyAsync(h, res, sizeof(h), cudaMemcpyDeviceToHost, a->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(a->stream);
   if (e != cudaSuccess) return cuda_fail(e, "sv_inner_product");
+  if ((st = take_pending_error(a)) != SV_OK || (st = take_pending_error(b)) != SV_OK) return st;
   if (a->prof) {
     a->d2h += sizeof(h);
     a->other_launches += a->n < 2 ? 1 : 2;

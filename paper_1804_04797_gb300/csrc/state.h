@@ -124,7 +124,7 @@ sv_status run_plan(sv_state *s, const svp::Plan &P, const svk::DevPlanView &view
 // (im); s is left unusable (the last pass did not write it).  *fused = false (and s
 // untouched) where these kernels are not in use for s's options or NVRTC is missing: the
 // caller then applies and reduces separately.
-sv_status apply_gates_inner(sv_state *s, const std::vector<svp::Gate> &g, const sv_state *with, double *out,
+sv_status apply_gates_inner(sv_state *s, const std::vector<svp::Gate> &g, sv_state *with, double *out,
                             bool *fused);
 // <g |x> | with> for each of the m basis states xs (re, im pairs in out), on plan-specialised
 // kernels that keep to the amplitudes which can differ from zero: outside the tile qubits of

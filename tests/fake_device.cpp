@@ -134,24 +134,32 @@ bool get_modules(const std::vector<const svp::Plan *> &p, int, std::vector<const
   return true;
 }
 cudaError_t prepare_passes(const Module *, const svp::Plan &) { return cudaSuccess; }
-namespace { cudaError_t pass() { queue([] {}); return cudaSuccess; } }
-cudaError_t launch_pass(const Module *, float2 *, int, const svk::DevPlanView &, int, const svp::DevPass &, cudaStream_t,
+// the plan kernels' launches, counted; the one with number g_fail gives up a wait
+int g_passes = 0, g_fail = -1;
+namespace {
+cudaError_t pass(const svk::DevPlanView &view) {
+  int *const err = g_passes++ == g_fail ? view.err : nullptr;
+  queue([err] { if (err) *err = 3; });
+  return cudaSuccess;
+}
+}  // namespace
+cudaError_t launch_pass(const Module *, float2 *, int, const svk::DevPlanView &view, int, const svp::DevPass &, cudaStream_t,
                         double *, unsigned *grid, const float2 *) {
   if (grid) *grid = 1;
-  return pass();
+  return pass(view);
 }
-cudaError_t launch_basis_pass(const Module *, float2 *, const svk::DevPlanView &, const svp::Plan &, int, uint64_t,
+cudaError_t launch_basis_pass(const Module *, float2 *, const svk::DevPlanView &view, const svp::Plan &, int, uint64_t,
                               cudaStream_t, double *, unsigned *grid, const float2 *) {
   if (grid) *grid = 1;
-  return pass();
+  return pass(view);
 }
-cudaError_t launch_fork_pass(const Module *, float2 *, const svk::DevPlanView &, const svp::Plan &, cudaStream_t) { return pass(); }
+cudaError_t launch_fork_pass(const Module *, float2 *, const svk::DevPlanView &view, const svp::Plan &, cudaStream_t) { return pass(view); }
 bool last_pass_tiles(const svp::Plan &, const std::vector<uint64_t> &needed, uint64_t, std::vector<uint64_t> *tiles) {
   *tiles = needed;
   return true;
 }
-cudaError_t launch_listed_pass(const Module *, float2 *, const svk::DevPlanView &, const svp::Plan &, const uint64_t *,
-                               size_t, cudaStream_t) { return pass(); }
+cudaError_t launch_listed_pass(const Module *, float2 *, const svk::DevPlanView &view, const svp::Plan &, const uint64_t *,
+                               size_t, cudaStream_t) { return pass(view); }
 }  // namespace svj
 
 // ---- scenarios ----------------------------------------------------------------------------
@@ -208,11 +216,35 @@ int uploads(int jit, int precision) {
   return g_copies < 12 || g_stale != 0;
 }
 
+// A wait that gave up in pass `fail` of a state: what the call says that reads the state.
+int gave_up(const std::string &how, int fail) {
+  sv_options o = options(1);
+  std::vector<double> out(4);
+  svj::g_fail = fail;
+  sv_status st = SV_OK;
+  if (how != "product") {  // the forward state of the inner-product amplitudes
+    if (how == "whole") o.pipeline = -1;  // (its backward states on whole passes)
+    const sv_lattice l = lattice(4, 4, 10, 5);
+    const uint64_t bits[2] = {1, 0x1234};
+    st = sv_amplitudes_by_inner_product(&l, 5, bits, 2, &o, out.data());
+  } else {
+    const std::vector<sv_gate> g = circuit(lattice(3, 4, 8, 5));
+    sv_state *s[2] = {nullptr, nullptr};
+    for (sv_state *&x : s)
+      if (!check(sv_create(12, &o, &x)) || !check(sv_apply_circuit(x, g.data(), g.size()))) return 2;
+    st = sv_inner_product(s[0], s[1], out.data());
+    for (sv_state *x : s) sv_destroy(x);
+  }
+  std::printf("status %d after %d passes\n", (int)st, svj::g_passes);
+  return st != (fail < 0 ? SV_OK : SV_ERR_TIMEOUT);
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
   const std::string what = argc > 1 ? argv[1] : "";
   auto arg = [&](int i) { return argc > i ? std::atoi(argv[i]) : 0; };
   if (what == "uploads") return uploads(arg(2), arg(3));
+  if (what == "gave_up") return gave_up(argc > 2 ? argv[2] : "", arg(3));
   return 3;
 }

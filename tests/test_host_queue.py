@@ -17,3 +17,10 @@ def test_sources_of_queued_copies_stay_as_they_are(fake_device, jit, precision):
     # (memory that is given back is overwritten at once)
     r = host_cpp.run(fake_device, 'uploads', jit, precision, env={'MALLOC_PERTURB_': '165'})
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize('how,passes', [('support', (0,)), ('whole', (0,)), ('product', (0, 3))])
+def test_a_state_that_was_not_finished_is_reported_by_the_call_that_reads_it(fake_device, how, passes):
+    for fail in (-1, *passes):
+        r = host_cpp.run(fake_device, 'gave_up', how, fail)
+        assert r.returncode == 0, r.stdout + r.stderr
