@@ -578,18 +578,19 @@ sv_status apply_gates(sv_state *s, const std::vector<svp::Gate> &g) {
   }
   if ((s->opts.precision == SV_PREC_TF32X3 || s->opts.precision == SV_PREC_F16X3) && !svk::fused_supported())
     return fail(SV_ERR_CUDA, "fused tensor-core path needs an sm_103a device");
-  if (g.empty() && !s->fresh) return SV_OK;
-  // the same gate list, options and starting condition as the last call: reuse its plan
+  if (g.empty() && !s->fresh) return s->fork > 0 ? fork_now(s) : SV_OK;
+  // the same gate list, options and starting condition as the last call: reuse its plan (one that
+  // forks a prefix or stores listed tiles serves one call)
   uint64_t key = 1469598103934665603ull;
   auto mix = [&key](const void *p, size_t len) {
     const unsigned char *b = static_cast<const unsigned char *>(p);
     for (size_t i = 0; i < len; ++i) key = (key ^ b[i]) * 1099511628211ull;
   };
-  const int head[10] = {s->n, s->fresh ? 1 : 0, s->opts.precision, s->opts.fuse_k, s->opts.tile_bits,
+  const int head[11] = {s->n, s->fresh ? 1 : 0, s->one_shape ? 1 : 0, s->opts.precision, s->opts.fuse_k, s->opts.tile_bits,
                         s->opts.low_bits, s->opts.jit, s->opts.pipeline, s->opts.norm_restore, s->opts.autotune};
   mix(head, sizeof(head));
   if (!g.empty()) mix(g.data(), g.size() * sizeof(svp::Gate));
-  if (s->plan_valid && s->plan_key == key) {
+  if (s->plan_valid && s->plan_key == key && s->fork == 0 && !s->needed) {
     const bool f16 = s->opts.precision == SV_PREC_F16X3;
     const bool kfused = s->plan_po.fused && !s->plan_jit;  // the tensor-core tile kernel
     if ((st = run_plan(s, s->plan, s->plan_view, kfused, f16, s->plan_jit)) != SV_OK) {
@@ -677,6 +678,7 @@ sv_status apply_gates(sv_state *s, const std::vector<svp::Gate> &g) {
   if ((st = run_plan(s, P, view, kfused, f16, jit)) != SV_OK) return st;
   s->fresh = false;
   if (kfused && (st = check_fused_error(s, view)) != SV_OK) return st;
+  if (P.fork > 0 || P.listed) return SV_OK;
   s->plan = std::move(P);
   s->plan_po = po;
   s->plan_jit = jit;

@@ -136,8 +136,10 @@ bool get_modules(const std::vector<const svp::Plan *> &p, int, std::vector<const
 cudaError_t prepare_passes(const Module *, const svp::Plan &) { return cudaSuccess; }
 // the plan kernels' launches, counted; the one with number g_fail gives up a wait
 int g_passes = 0, g_fail = -1;
+std::string g_kinds;  // w(hole), b(asis), f(ork), l(isted)
 namespace {
-cudaError_t pass(const svk::DevPlanView &view) {
+cudaError_t pass(char kind, const svk::DevPlanView &view) {
+  g_kinds += kind;
   int *const err = g_passes++ == g_fail ? view.err : nullptr;
   queue([err] { if (err) *err = 3; });
   return cudaSuccess;
@@ -146,20 +148,20 @@ cudaError_t pass(const svk::DevPlanView &view) {
 cudaError_t launch_pass(const Module *, float2 *, int, const svk::DevPlanView &view, int, const svp::DevPass &, cudaStream_t,
                         double *, unsigned *grid, const float2 *) {
   if (grid) *grid = 1;
-  return pass(view);
+  return pass('w', view);
 }
 cudaError_t launch_basis_pass(const Module *, float2 *, const svk::DevPlanView &view, const svp::Plan &, int, uint64_t,
                               cudaStream_t, double *, unsigned *grid, const float2 *) {
   if (grid) *grid = 1;
-  return pass(view);
+  return pass('b', view);
 }
-cudaError_t launch_fork_pass(const Module *, float2 *, const svk::DevPlanView &view, const svp::Plan &, cudaStream_t) { return pass(view); }
+cudaError_t launch_fork_pass(const Module *, float2 *, const svk::DevPlanView &view, const svp::Plan &, cudaStream_t) { return pass('f', view); }
 bool last_pass_tiles(const svp::Plan &, const std::vector<uint64_t> &needed, uint64_t, std::vector<uint64_t> *tiles) {
   *tiles = needed;
   return true;
 }
 cudaError_t launch_listed_pass(const Module *, float2 *, const svk::DevPlanView &view, const svp::Plan &, const uint64_t *,
-                               size_t, cudaStream_t) { return pass(view); }
+                               size_t, cudaStream_t) { return pass('l', view); }
 }  // namespace svj
 
 // ---- scenarios ----------------------------------------------------------------------------
@@ -239,6 +241,29 @@ int gave_up(const std::string &how, int fail) {
   return st != (fail < 0 ? SV_OK : SV_ERR_TIMEOUT);
 }
 
+// One gate list on a handle as a tree's segment (forking its prefix, or storing listed tiles), as a
+// whole state, and as a segment again; and the fork of an empty list.
+int segments() {
+  const sv_options o = options(1);
+  sv_state *s = nullptr;
+  if (!check(sv_create(12, &o, &s))) return 2;
+  s->fresh = false;
+  const std::vector<svp::Gate> g = {svp::Gate{svp::K_SX, 3, 0}};
+  const std::vector<uint64_t> needed = {5};
+  auto apply = [&](int fork, bool listed, const std::vector<svp::Gate> &list) {
+    s->fork = fork;
+    s->needed = listed ? &needed : nullptr;
+    const bool ok = check(svc::apply_gates(s, list));
+    s->needed = nullptr;
+    return ok && s->fork == 0;
+  };
+  const bool ok = apply(1, false, g) && apply(0, false, g) && apply(0, true, g) && apply(0, false, g) &&
+                  apply(0, false, g) && apply(1, false, g) && apply(0, true, g) && apply(1, false, {});
+  sv_destroy(s);
+  std::printf("passes %s\n", svj::g_kinds.c_str());
+  return !ok || svj::g_kinds != "fwlwwfl";
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -246,5 +271,6 @@ int main(int argc, char **argv) {
   auto arg = [&](int i) { return argc > i ? std::atoi(argv[i]) : 0; };
   if (what == "uploads") return uploads(arg(2), arg(3));
   if (what == "gave_up") return gave_up(argc > 2 ? argv[2] : "", arg(3));
+  if (what == "segments") return segments();
   return 3;
 }

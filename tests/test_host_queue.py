@@ -24,3 +24,8 @@ def test_a_state_that_was_not_finished_is_reported_by_the_call_that_reads_it(fak
     for fail in (-1, *passes):
         r = host_cpp.run(fake_device, 'gave_up', how, fail)
         assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_a_segment_s_plan_serves_no_other_call(fake_device):
+    r = host_cpp.run(fake_device, 'segments')
+    assert r.returncode == 0, r.stdout + r.stderr
