@@ -124,6 +124,7 @@ struct JitCircuit {
 // Everything one batch needs on the device, plus its instantiated graph.
 struct Batch {
   std::string key;
+  int device = 0;
   int m = 13;
   int count = 0;
   std::vector<int> nq;
@@ -143,6 +144,17 @@ struct Batch {
     if (stream) cudaStreamDestroy(stream);
     for (cudaStream_t b : branch) cudaStreamDestroy(b);
     for (cudaEvent_t e : ev) cudaEventDestroy(e);
+  }
+};
+
+// The calling thread's current device is `device` while this lives.
+struct OnDevice {
+  int was = -1;
+  explicit OnDevice(int device) {
+    if (cudaGetDevice(&was) != cudaSuccess || was == device || cudaSetDevice(device) != cudaSuccess) was = -1;
+  }
+  ~OnDevice() {
+    if (was >= 0) cudaSetDevice(was);
   }
 };
 
@@ -255,6 +267,7 @@ sv_status build_jit_circuits(const std::vector<std::vector<svp::Gate>> &gates, c
 // Build plans, the work queue and the device buffers of a batch with tile size m.
 sv_status build_batch(const sv_lattice *circs, size_t count, int m_req, int jit, Batch *B) {
   B->count = (int)count;
+  cudaGetDevice(&B->device);
   B->nq.resize(count);
   int n_min = 64;  // smallest circuit (of the persistent launch, below)
   std::vector<std::vector<svp::Gate>> gates(count);
@@ -539,6 +552,7 @@ extern "C" sv_status sv_batch_amplitudes(size_t circuit, const uint64_t *bits, s
   // circuits 1.36 ms, now 1.11)
   const float2 *psi = static_cast<const float2 *>(g_batch->states.p) + off;
   float2 *picked = static_cast<float2 *>(g_batch->picked.p);
+  const OnDevice on(g_batch->device);  // (a kernel reads them: the thread may be on another device by now)
   for (size_t j0 = 0; j0 < m; j0 += svk::kPickMost) {
     const size_t k = std::min<size_t>(m - j0, svk::kPickMost);
     svk::PickArgs args;

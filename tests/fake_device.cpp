@@ -21,6 +21,7 @@
 namespace {
 std::deque<std::function<void()>> g_queue;
 size_t g_done = 0, g_queued = 0;
+int g_device = 0;
 int g_stale = 0, g_copies = 0;  // copies whose source was not what it was when they were queued
 
 void queue(std::function<void()> f) {
@@ -73,8 +74,8 @@ cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t) { *reinterpret_cast<siz
 cudaError_t cudaEventSynchronize(cudaEvent_t e) { drain(*reinterpret_cast<size_t *>(e)); return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { *ms = 1.f; return cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t e) { delete reinterpret_cast<size_t *>(e); return cudaSuccess; }
-cudaError_t cudaGetDevice(int *d) { *d = 0; return cudaSuccess; }
-cudaError_t cudaSetDevice(int) { return cudaSuccess; }
+cudaError_t cudaGetDevice(int *d) { *d = g_device; return cudaSuccess; }
+cudaError_t cudaSetDevice(int d) { g_device = d; return cudaSuccess; }
 cudaError_t cudaGetDeviceProperties(cudaDeviceProp *p, int) { std::memset(p, 0, sizeof(*p)); return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 const char *cudaGetErrorString(cudaError_t) { return "error"; }
@@ -109,7 +110,8 @@ cudaError_t launch_batch_items(const BatchCP *, uint32_t, BatchItem *, uint32_t,
 int batch_run_log(uint32_t, double) { return 0; }
 int batch_grid(uint32_t, int) { return 152; }
 cudaError_t launch_batch(float2 *, const unsigned char *, uint32_t, const BatchCP *, const BatchItem *, uint32_t, unsigned *, int, cudaStream_t, unsigned long long, int) { return nothing(); }
-cudaError_t launch_pick(const float2 *, const PickArgs &, int, float2 *, cudaStream_t) { return nothing(); }
+int g_picked_on = -1;
+cudaError_t launch_pick(const float2 *, const PickArgs &, int, float2 *, cudaStream_t) { g_picked_on = g_device; return nothing(); }
 cudaError_t launch_batch_stats(const float2 *, const BatchChunk *, int, double *, const int *, int, double *, cudaStream_t) { return nothing(); }
 }  // namespace svk
 namespace svc {
@@ -264,6 +266,19 @@ int segments() {
   return !ok || svj::g_kinds != "fwlwwfl";
 }
 
+// Amplitudes of a batch, read while the thread's current device is another one.
+int other_device() {
+  const sv_lattice l = lattice(3, 4, 8, 5);
+  const uint64_t bits[2] = {1, 2};
+  double out[4];
+  g_device = 1;
+  if (!check(sv_apply_batch(&l, 1, nullptr, nullptr))) return 2;
+  g_device = 0;
+  if (!check(sv_batch_amplitudes(0, bits, 2, out))) return 2;
+  std::printf("picked on device %d, left on %d\n", svk::g_picked_on, g_device);
+  return svk::g_picked_on != 1 || g_device != 0;
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -272,5 +287,6 @@ int main(int argc, char **argv) {
   if (what == "uploads") return uploads(arg(2), arg(3));
   if (what == "gave_up") return gave_up(argc > 2 ? argv[2] : "", arg(3));
   if (what == "segments") return segments();
+  if (what == "other_device") return other_device();
   return 3;
 }

@@ -29,3 +29,8 @@ def test_a_state_that_was_not_finished_is_reported_by_the_call_that_reads_it(fak
 def test_a_segment_s_plan_serves_no_other_call(fake_device):
     r = host_cpp.run(fake_device, 'segments')
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_a_batch_s_amplitudes_are_read_on_its_device(fake_device):
+    r = host_cpp.run(fake_device, 'other_device')
+    assert r.returncode == 0, r.stdout + r.stderr
