@@ -59,7 +59,8 @@ __device__ __forceinline__ uint64_t spread(uint64_t i, const uint8_t *bit, int n
 
 // Operand images.  Aop: slice s of B, row tile rt, chunk kc at (((s * rtiles + rt) * kch + kc) *
 // 2 + part) * kABlock; Bop likewise with A, its column tiles and kBBlock.  One thread per
-// (slice, row, k) of each operand.
+// (slice, row, k) of each operand.  FIXED: as below.
+template <bool FIXED>
 __global__ void outer_prep_kernel(const float2 *__restrict__ A, const float2 *__restrict__ B, const OuterShape S,
                                   int kch, unsigned char *__restrict__ aimg, unsigned char *__restrict__ bimg) {
   const uint64_t L = 1ull << S.t, K = (uint64_t)kch * kKc;
@@ -71,8 +72,8 @@ __global__ void outer_prep_kernel(const float2 *__restrict__ A, const float2 *__
     unsigned char *dst;
     uint32_t blk;
     if (e < nA_ops) {  // Aop[row, k] of slice row / nb
-      const uint64_t row = e / K, k = e % K, l = k >> 1, slice = row >> S.nB;
-      const uint64_t xb = spread(row & (nb - 1), S.b_bit, S.nB);
+      const uint64_t row = e / K, k = e % K, l = k >> 1, slice = FIXED ? row >> S.nB : 0;
+      const uint64_t xb = FIXED ? spread(row & (nb - 1), S.b_bit, S.nB) : row;
       const float2 z = l < L ? B[xb + (l << S.nB) + (slice << (S.nB + S.t))] : make_float2(0.f, 0.f);
       v = (k & 1) ? z.y : z.x;
       const uint64_t rt = row / kRows, kc = k / kKc;
@@ -83,8 +84,8 @@ __global__ void outer_prep_kernel(const float2 *__restrict__ A, const float2 *__
       *reinterpret_cast<float *>(dst + o) = h;
       *reinterpret_cast<float *>(dst + blk + o) = tf32_rn(v - h);
     } else {  // Bop[n, k], n = 2 column + o, of slice column / na
-      const uint64_t f = e - nA_ops, n = f / K, k = f % K, l = k >> 1, slice = (n >> 1) >> S.nA;
-      const uint64_t xa = spread((n >> 1) & (na - 1), S.a_bit, S.nA);
+      const uint64_t f = e - nA_ops, n = f / K, k = f % K, l = k >> 1, slice = FIXED ? (n >> 1) >> S.nA : 0;
+      const uint64_t xa = FIXED ? spread((n >> 1) & (na - 1), S.a_bit, S.nA) : n >> 1;
       const float2 z = l < L ? A[xa + (l << S.nA) + (slice << (S.nA + S.t))] : make_float2(0.f, 0.f);
       const bool im_out = n & 1, im_in = k & 1;
       v = !im_out ? (im_in ? -z.y : z.x) : (im_in ? z.x : z.y);
@@ -130,6 +131,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
   return false;
 }
 
+// FIXED: some branches are fixed by output bits, so that a tile's rows and columns lie in
+// OuterShape's order (else in the state's: one address per row).  SCALED: with signs, or a scale
+// with a lo part.  A product that needs neither (every expanded CZ summed over) keeps to one
+// multiplication a value and a running address, and its operands' images to the state's order.
+// Both kernels with one form for all / with these, us at 28 qubits on one GB300: 2^7 branches
+// summed 1415 / 1355, 2^4 and three signs 696 / 640, 2^5 and two more fixed 644 / 645.
+template <bool FIXED, bool SCALED>
 __global__ void __launch_bounds__(128, 2)
 outer_mma_kernel(const unsigned char *__restrict__ aimg, const unsigned char *__restrict__ bimg, int rtiles, int ctiles,
                  int kch, const OuterShape S, float2 scale, float2 *__restrict__ out, int *err) {
@@ -141,8 +149,10 @@ outer_mma_kernel(const unsigned char *__restrict__ aimg, const unsigned char *__
   __shared__ int stop;
   __shared__ uint64_t col_at[kCols], row_at[kRows];  // x_A of a tile's columns, x_B of its rows
   const int tid = threadIdx.x, warp = tid >> 5, nA = S.nA;
-  col_at[tid] = spread(tid, S.a_bit, 7);
-  row_at[tid] = spread(tid, S.b_bit, 7);
+  if (FIXED || SCALED) {
+    col_at[tid] = FIXED ? spread(tid, S.a_bit, 7) : tid;
+    row_at[tid] = FIXED ? spread(tid, S.b_bit, 7) : tid;
+  }
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&load_bar)));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mma_bar)));
@@ -162,11 +172,14 @@ outer_mma_kernel(const unsigned char *__restrict__ aimg, const unsigned char *__
   const uint64_t ntiles = (uint64_t)rtiles * ctiles;
   for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const uint64_t rt = tile / ctiles, ct = tile % ctiles;
-    const uint64_t xa0 = spread(ct * kCols, S.a_bit, nA), xb0 = spread(rt * kRows, S.b_bit, S.nB);
+    const uint64_t xa0 = FIXED ? spread(ct * kCols, S.a_bit, nA) : ct * kCols;
+    const uint64_t xb0 = FIXED ? spread(rt * kRows, S.b_bit, S.nB) : rt * kRows;
     // the slices that the tile's fixed bits select
     uint64_t slice_a = 0, slice_b = 0;
-    for (int j = 0; j < S.fix_a; ++j) slice_a |= ((xb0 >> S.fix_a_by[j]) & 1ull) << j;
-    for (int j = 0; j < S.fix_b; ++j) slice_b |= ((xa0 >> S.fix_b_by[j]) & 1ull) << j;
+    if (FIXED) {
+      for (int j = 0; j < S.fix_a; ++j) slice_a |= ((xb0 >> S.fix_a_by[j]) & 1ull) << j;
+      for (int j = 0; j < S.fix_b; ++j) slice_b |= ((xa0 >> S.fix_b_by[j]) & 1ull) << j;
+    }
     for (int kc = 0; kc < kch; ++kc) {
       if (tid == 0) {
         const uint32_t lb = smem_u32(&load_bar);
@@ -221,12 +234,17 @@ outer_mma_kernel(const unsigned char *__restrict__ aimg, const unsigned char *__
     const int lane = tid & 31;
     // the absorbed CZs' signs: the bits of x_A whose parity is this lane's row's sign
     uint64_t sign_mask = 0;
-    for (int j = 0; j < S.signs; ++j)
-      sign_mask ^= (((xb0 + row_at[32 * warp + lane]) >> S.sign_b[j]) & 1ull) << S.sign_a[j];
+    if (SCALED)
+      for (int j = 0; j < S.signs; ++j)
+        sign_mask ^= (((xb0 + row_at[32 * warp + lane]) >> S.sign_b[j]) & 1ull) << S.sign_a[j];
     const uint32_t sign_base = __popcll(sign_mask & xa0);
     float4 *stg = reinterpret_cast<float4 *>(sa) + warp * 256;
-    const bool neighbours = S.a_bit[0] == 0;
-    auto scaled = [&](uint32_t v) { return fmaf(__uint_as_float(v), scale.x, __uint_as_float(v) * scale.y); };
+    float2 *const rows = out + ((xb0 + (uint64_t)(32 * warp)) << nA) + xa0;
+    const bool neighbours = !FIXED || S.a_bit[0] == 0;
+    auto scaled = [&](uint32_t v) {
+      const float x = __uint_as_float(v);
+      return SCALED ? fmaf(x, scale.x, x * scale.y) : x * scale.x;
+    };
 #pragma unroll 1
     for (int c = 0; c < 256; c += 32) {
       uint32_t r[32];
@@ -240,7 +258,7 @@ outer_mma_kernel(const unsigned char *__restrict__ aimg, const unsigned char *__
           : "r"(taddr + (uint32_t)c)
           : "memory");
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      if (sign_mask) {
+      if (SCALED && sign_mask) {
 #pragma unroll
         for (int q = 0; q < 32; ++q)  // (column c / 2 + q / 2 of the tile)
           r[q] ^= (sign_base + __popcll(sign_mask & col_at[c / 2 + q / 2])) << 31;
@@ -254,7 +272,8 @@ outer_mma_kernel(const unsigned char *__restrict__ aimg, const unsigned char *__
       for (int q = 0; q < 8; ++q) {
         const int row = 4 * q + (lane >> 3), ch = lane & 7;
         const float4 v = stg[row * 8 + (ch ^ (row & 7))];
-        float2 *const to = out + ((xb0 + row_at[32 * warp + row]) << nA) + xa0 + col_at[c / 2 + 2 * ch];
+        float2 *const to = FIXED ? out + ((xb0 + row_at[32 * warp + row]) << nA) + xa0 + col_at[c / 2 + 2 * ch]
+                                 : rows + ((uint64_t)row << nA) + c / 2 + 2 * ch;
         if (neighbours) {
           *reinterpret_cast<float4 *>(to) = v;
         } else {
@@ -295,12 +314,16 @@ size_t outer_sum_tc_scratch(const OuterShape &S) {
 cudaError_t launch_outer_sum_tc(const float2 *A, const float2 *B, const OuterShape &S, float2 scale, float2 *out,
                                 void *scratch, int *err, cudaStream_t st) {
   if (!outer_sum_tc_supported(S)) return cudaErrorInvalidValue;
-  static bool configured = false;
-  if (!configured) {
+  const int form = S.fix_a + S.fix_b > 0 ? 2 : S.signs > 0 || scale.y != 0.f ? 1 : 0;
+  const auto kernel = form == 0   ? outer_mma_kernel<false, false>
+                      : form == 1 ? outer_mma_kernel<false, true>
+                                  : outer_mma_kernel<true, true>;
+  static bool configured[3] = {};
+  if (!configured[form]) {
     const cudaError_t e =
-        cudaFuncSetAttribute(outer_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem + 1024);
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem + 1024);
     if (e != cudaSuccess) return e;
-    configured = true;
+    configured[form] = true;
   }
   const int kch = (int)(((2ull << S.t) + kKc - 1) / kKc);
   const int rtiles = (int)((1ull << S.nB) / kRows), ctiles = (int)((1ull << S.nA) / kCols);
@@ -310,13 +333,13 @@ cudaError_t launch_outer_sum_tc(const float2 *A, const float2 *B, const OuterSha
   uint64_t pgrid = (work + 255) / 256;
   const uint64_t pmax = (uint64_t)device_sm_count() * 8;
   if (pgrid > pmax) pgrid = pmax;
-  outer_prep_kernel<<<(unsigned)pgrid, 256, 0, st>>>(A, B, S, kch, aimg, bimg);
+  (form == 2 ? outer_prep_kernel<true> : outer_prep_kernel<false>)<<<(unsigned)pgrid, 256, 0, st>>>(A, B, S, kch, aimg, bimg);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   uint64_t grid = (uint64_t)device_sm_count() * 2;
   const uint64_t ntiles = (uint64_t)rtiles * ctiles;
   if (grid > ntiles) grid = ntiles;
-  outer_mma_kernel<<<(unsigned)grid, 128, kSmem + 1024, st>>>(aimg, bimg, rtiles, ctiles, kch, S, scale, out, err);
+  kernel<<<(unsigned)grid, 128, kSmem + 1024, st>>>(aimg, bimg, rtiles, ctiles, kch, S, scale, out, err);
   return cudaGetLastError();
 }
 
