@@ -252,7 +252,9 @@ sv_status sv_branch_amplitudes(const sv_lattice *lat, const sv_cut *cut, const u
  * accumulation).  Unless cut->full_decomposition: the product applies the signs of crossing
  * CZs that only sign the output, and an implicit decomposition (see sv_branch_amplitudes)
  * fixes its branch by an output bit for a whole tile of the product, so only the others are
- * summed over (at least 7 bits of either half stay free of them).  Half A must be qubits
+ * summed over (at least 7 bits of either half stay free of them).  The tensor-core precisions
+ * form the product on the tensor cores, or on the CUDA cores where halves of fewer than 7
+ * qubits or too little memory for its operands leave no choice.  Half A must be qubits
  * 0..n_A-1 (a cut between lattice rows).  SV_ERR_ARG otherwise. */
 sv_status sv_branch_full_state(const sv_lattice *lat, const sv_cut *cut, const sv_options *opts, sv_state *out);
 

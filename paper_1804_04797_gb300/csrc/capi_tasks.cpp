@@ -485,18 +485,22 @@ extern "C" sv_status sv_branch_full_state(const sv_lattice *lat, const sv_cut *c
     S.sign_b[S.signs++] = (uint8_t)(odd[i].second - C.na);
   }
   // the tensor-core precisions: the product on tcgen05 (TF32x3), else on the CUDA cores
-  const bool tc = (o.precision == SV_PREC_TF32X3 || o.precision == SV_PREC_F16X3) &&
-                  svk::fused_supported() && svk::outer_sum_tc_supported(S);
+  bool tc = (o.precision == SV_PREC_TF32X3 || o.precision == SV_PREC_F16X3) && svk::fused_supported() &&
+            svk::outer_sum_tc_supported(S);
   void *scratch = nullptr;
   int *d_err = nullptr;
+  // also on the CUDA cores (which need no memory beside the halves) where the operand images find no
+  // room: fixed branches take an image for each combination of them, of 16 branches at least, so
+  // that the images can be many times those of the whole decomposition (no branch summed over, six
+  // fixed on one side: 16 times)
+  if (e == cudaSuccess && tc && cudaMalloc(&scratch, svk::outer_sum_tc_scratch(S) + 256) != cudaSuccess) {
+    cudaGetLastError();
+    scratch = nullptr;
+    tc = false;
+  }
   if (e == cudaSuccess && tc) {
-    e = cudaMalloc(&scratch, svk::outer_sum_tc_scratch(S) + 256);
-    if (e == cudaSuccess) {
-      d_err = reinterpret_cast<int *>(static_cast<char *>(scratch) + svk::outer_sum_tc_scratch(S));
-      e = cudaMemsetAsync(d_err, 0, sizeof(int), out->stream);
-    } else {
-      scratch = nullptr;
-    }
+    d_err = reinterpret_cast<int *>(static_cast<char *>(scratch) + svk::outer_sum_tc_scratch(S));
+    e = cudaMemsetAsync(d_err, 0, sizeof(int), out->stream);
     if (e == cudaSuccess) {
       profile_begin(out);
       e = svk::launch_outer_sum_tc(A.s->psi, B.s->psi, S, scale, out->psi, scratch, d_err, out->stream);

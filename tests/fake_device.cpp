@@ -40,7 +40,11 @@ void drain(size_t until = ~(size_t)0) {
 
 // ---- runtime ----------------------------------------------------------------------------
 extern "C" {
-cudaError_t cudaMalloc(void **p, size_t n) { *p = std::calloc(1, n); return *p ? cudaSuccess : cudaErrorMemoryAllocation; }
+cudaError_t cudaMalloc(void **p, size_t n) {
+  if (n > 1ull << 40) { *p = nullptr; return cudaErrorMemoryAllocation; }
+  *p = std::calloc(1, n);
+  return *p ? cudaSuccess : cudaErrorMemoryAllocation;
+}
 cudaError_t cudaFree(void *p) { drain(); std::free(p); return cudaSuccess; }
 cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) { drain(); std::memcpy(d, s, n); return cudaSuccess; }
 cudaError_t cudaMemset(void *d, int v, size_t n) { drain(); std::memset(d, v, n); return cudaSuccess; }
@@ -100,9 +104,11 @@ cudaError_t launch_gather_prob(const float2 *, const uint64_t *, int64_t, double
 cudaError_t launch_branch_gather(const float2 *, int, int, const uint64_t *, uint64_t, float2 *, cudaStream_t) { return nothing(); }
 cudaError_t launch_branch_sum(const float2 *, int, const float2 *, int, int, const uint64_t *, const uint64_t *, int, double, double *, cudaStream_t) { return nothing(); }
 cudaError_t launch_fork(float2 *, int, int, cudaStream_t) { return nothing(); }
-cudaError_t launch_outer_sum(const float2 *, const float2 *, const OuterShape &, float2, float2 *, cudaStream_t) { return nothing(); }
-bool outer_sum_tc_supported(const OuterShape &) { return false; }
-size_t outer_sum_tc_scratch(const OuterShape &) { return 0; }
+int g_outer = 0;
+bool g_outer_tc = false;
+cudaError_t launch_outer_sum(const float2 *, const float2 *, const OuterShape &, float2, float2 *, cudaStream_t) { ++g_outer; return nothing(); }
+bool outer_sum_tc_supported(const OuterShape &) { return g_outer_tc; }
+size_t outer_sum_tc_scratch(const OuterShape &) { return (size_t)1 << 41; }
 cudaError_t launch_outer_sum_tc(const float2 *, const float2 *, const OuterShape &, float2, float2 *, void *, int *, cudaStream_t) { return nothing(); }
 cudaError_t launch_inner(const float2 *, const float2 *, int, double *, double *, cudaStream_t) { return nothing(); }
 cudaError_t launch_basis_state(float2 *, int, uint64_t, cudaStream_t) { return nothing(); }
@@ -279,6 +285,21 @@ int other_device() {
   return svk::g_picked_on != 1 || g_device != 0;
 }
 
+// The full state from two halves on the tensor cores, whose operand images find no room.
+int no_room() {
+  const sv_options o = options(0, SV_PREC_TF32X3);
+  sv_cut cut;
+  std::memset(&cut, 0, sizeof(cut));
+  cut.half_a_mask = 0xff;
+  const sv_lattice l = lattice(4, 4, 8, 5);
+  sv_state *s = nullptr;
+  svk::g_outer_tc = true;
+  if (!check(sv_create(16, &o, &s))) return 2;
+  const bool ok = check(sv_branch_full_state(&l, &cut, &o, s));
+  sv_destroy(s);
+  return !ok || svk::g_outer != 1;
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -288,5 +309,6 @@ int main(int argc, char **argv) {
   if (what == "gave_up") return gave_up(argc > 2 ? argv[2] : "", arg(3));
   if (what == "segments") return segments();
   if (what == "other_device") return other_device();
+  if (what == "no_room") return no_room();
   return 3;
 }

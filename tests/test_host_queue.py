@@ -34,3 +34,8 @@ def test_a_segment_s_plan_serves_no_other_call(fake_device):
 def test_a_batch_s_amplitudes_are_read_on_its_device(fake_device):
     r = host_cpp.run(fake_device, 'other_device')
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_the_tensor_form_runs_where_its_operand_images_find_no_room(fake_device):
+    r = host_cpp.run(fake_device, 'no_room')
+    assert r.returncode == 0, r.stdout + r.stderr
