@@ -1237,8 +1237,20 @@ void write_file(const std::string &path, const std::string &data) {
 
 namespace {
 
+// The texts of the headers that every source includes: part of a cached cubin's key, as the source
+// itself does not change with them.
+const std::string &headers_key() {
+  static const std::string key = [] {
+    std::string all;
+    for (int i = 0; i < kHeaderCount; ++i) all += std::string(kHeaderNames[i]) + '\n' + kHeaderSources[i];
+    return std::to_string(fnv1a(all));
+  }();
+  return key;
+}
+
 // Compile sources to cubins in a pool of one worker per hardware thread; a cubin whose
-// source hash is in the cache directory is read instead.  ok[i] = 0 where NVRTC failed.
+// key (source, headers, architecture) is in the cache directory is read instead.  ok[i] = 0
+// where NVRTC failed.
 void compile_sources(const std::vector<std::string> &src, const char *arch, const std::string &cache,
                      std::vector<std::string> *cubins, std::vector<std::string> *logs, std::vector<char> *ok) {
   const size_t ns = src.size();
@@ -1250,7 +1262,7 @@ void compile_sources(const std::vector<std::string> &src, const char *arch, cons
   for (size_t i = 0; i < ns; ++i) {
     if (!cache.empty()) {
       char name[96];
-      std::snprintf(name, sizeof(name), "/%016llx_%s.cubin", (unsigned long long)fnv1a(src[i] + arch), arch);
+      std::snprintf(name, sizeof(name), "/%016llx_%s.cubin", (unsigned long long)fnv1a(src[i] + headers_key() + arch), arch);
       file[i] = cache + name;
       if (read_file(file[i], &(*cubins)[i])) continue;
     }

@@ -70,7 +70,7 @@ std::string pass_source(const svp::Plan &P, int kpr, int pass, bool inner = fals
 bool compile(const std::string &src, const char *arch, std::string *cubin, std::string *log);
 
 // Compile the kernels of every pass of a plan (one NVRTC program per pass, in parallel
-// threads).  cache: a directory of cubins by source hash ("" = none).
+// threads).  cache: a directory of cubins by the hash of their source and headers ("" = none).
 bool compile_plan(const svp::Plan &P, int kpr, const char *arch, std::vector<std::string> *cubins,
                   std::string *log, const std::string &cache);
 

@@ -7,11 +7,12 @@ CSRC = os.path.join(ROOT, 'paper_1804_04797_gb300', 'csrc')
 CUDA = os.environ.get('CUDA_HOME', '/usr/local/cuda')
 
 
-def build(out_dir, program, sources):
-    """tests/<program>.cpp with library sources, as an executable in out_dir."""
+def build(out_dir, program, sources, more=()):
+    """tests/<program>.cpp with library sources, as an executable in out_dir (more: further files and
+    flags)."""
     exe = os.path.join(str(out_dir), program)
     cmd = ['g++', '-std=c++17', '-O1', '-I', CSRC, '-I', os.path.join(CUDA, 'include'), '-o', exe,
-           os.path.join(ROOT, 'tests', program + '.cpp')] + [os.path.join(CSRC, s) for s in sources] + ['-ldl', '-lpthread']
+           os.path.join(ROOT, 'tests', program + '.cpp')] + [os.path.join(CSRC, s) for s in sources] + list(more) + ['-ldl', '-lpthread']
     r = subprocess.run(cmd, capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
     return exe
