@@ -71,9 +71,11 @@ enum {
 /* Options.  Zero-initialised fields take the defaults in brackets. */
 typedef struct {
   int fuse_k;     /* qubits per register group besides qubit 0 (plain) or per fused   */
-                  /* block (tensor cores), 1..5; 0 = the default 5 (the plain kernels  */
-                  /* use at most 4).  The tensor-core precisions    */
-                  /* take 5 (32x32 stage unitaries) or 4 (16x16, 12-qubit tiles only);  */
+                  /* block (tensor cores), 1..5; 0 = the default: 5 on the tensor      */
+                  /* cores, 4 on the plain kernels (which use at most 4), but 2 on the */
+                  /* interpreting kernel for states of at most 11 and of 13..15 qubits */
+                  /* (with tile_bits and low_bits 0 too).  The tensor-core precisions  */
+                  /* take 5 (32x32 stage unitaries) or 4 (16x16, 12-qubit tiles only); */
                   /* any other value is SV_ERR_ARG.                                    */
   int precision;  /* SV_PREC_*                                            [PLAIN]       */
   int autotune;   /* 1 = pick shapes by timing, kept in a JSON cache (SV_AUTOTUNE_CACHE, */

@@ -37,15 +37,12 @@ using PRegs = P2[1 << RK];
 #define SVG_PAIRS_4_1(M) M(0, 2) M(1, 3) M(4, 6) M(5, 7) M(8, 10) M(9, 11) M(12, 14) M(13, 15)
 #define SVG_PAIRS_4_2(M) M(0, 4) M(1, 5) M(2, 6) M(3, 7) M(8, 12) M(9, 13) M(10, 14) M(11, 15)
 #define SVG_PAIRS_4_3(M) M(0, 8) M(1, 9) M(2, 10) M(3, 11) M(4, 12) M(5, 13) M(6, 14) M(7, 15)
-#define SVG_PAIRS_3_0(M) M(0, 1) M(2, 3) M(4, 5) M(6, 7)
-#define SVG_PAIRS_3_1(M) M(0, 2) M(1, 3) M(4, 6) M(5, 7)
-#define SVG_PAIRS_3_2(M) M(0, 4) M(1, 5) M(2, 6) M(3, 7)
 #define SVG_PAIRS_2_0(M) M(0, 1) M(2, 3)
 #define SVG_PAIRS_2_1(M) M(0, 2) M(1, 3)
 // (all pairs)
 #define SVG_ALL_2(M) M(0) M(1) M(2) M(3)
-#define SVG_ALL_3(M) SVG_ALL_2(M) M(4) M(5) M(6) M(7)
-#define SVG_ALL_4(M) SVG_ALL_3(M) M(8) M(9) M(10) M(11) M(12) M(13) M(14) M(15)
+#define SVG_ALL_4(M) \
+  SVG_ALL_2(M) M(4) M(5) M(6) M(7) M(8) M(9) M(10) M(11) M(12) M(13) M(14) M(15)
 
 // The next op: its words were read ahead; read the one after it.
 #define SVG_NEXT                                  \
@@ -169,25 +166,6 @@ __device__ __forceinline__ void run_gates<2>(PRegs<2> &R, PRegs<2> &I, uint32_t 
       : "memory");
 }
 #undef SVG_IO_2
-
-#define SVG_IO_3(M) M(0, 0, 8) M(1, 1, 9) M(2, 2, 10) M(3, 3, 11) M(4, 4, 12) M(5, 5, 13) M(6, 6, 14) M(7, 7, 15)
-template <>
-__device__ __forceinline__ void run_gates<3>(PRegs<3> &R, PRegs<3> &I, uint32_t at, uint32_t W) {
-  asm volatile(
-      SVG_HEAD SVG_ALL_3(SVG_DECL) SVG_IO_3(SVG_IN) "mov.b32 at, %16; mov.b32 W, %17;\n" SVG_CONSTANTS
-      "TS: .branchtargets IM0, IM1, IM2, IM0, IM4, RE0, RE1, RE2, RE0, RE4, H0, H1, H2, H0, H4, T0, T1, T2, T0, T4,"
-      " S0, S1, S2, S0, S4, C0, C1, C0, C3, C0, C0, CP0, CP1, CP2, CP0, RS, END;\n" SVG_START
-      SVG_SLOT(0, SVG_PAIRS_3_0) SVG_SLOT(1, SVG_PAIRS_3_1) SVG_SLOT(2, SVG_PAIRS_3_2) SVG_PACKSLOT(SVG_ALL_3)
-      "C0: " SVG_NEG(3) SVG_NEG(7) SVG_NEXT
-      "C1: " SVG_NEG(5) SVG_NEG(7) SVG_NEXT
-      "C3: " SVG_NEG(6) SVG_NEG(7) SVG_NEXT
-      "END:\n" SVG_IO_3(SVG_OUT) "}\n"
-      : "+l"(R[0]), "+l"(R[1]), "+l"(R[2]), "+l"(R[3]), "+l"(R[4]), "+l"(R[5]), "+l"(R[6]), "+l"(R[7]), "+l"(I[0]),
-        "+l"(I[1]), "+l"(I[2]), "+l"(I[3]), "+l"(I[4]), "+l"(I[5]), "+l"(I[6]), "+l"(I[7])
-      : "r"(at), "r"(W)
-      : "memory");
-}
-#undef SVG_IO_3
 
 #define SVG_IO_4(M)                                                                                          \
   M(0, 0, 16) M(1, 1, 17) M(2, 2, 18) M(3, 3, 19) M(4, 4, 20) M(5, 5, 21) M(6, 6, 22) M(7, 7, 23) M(8, 8, 24) \

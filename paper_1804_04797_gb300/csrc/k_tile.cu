@@ -7,7 +7,7 @@
 // 16-byte vector).  The tile is staged in shared memory (the on-chip copy of the
 // paper's "local qubits" in LDM, §2.3) and every gate of the pass is applied to it:
 // stage by stage, each thread pulls the amplitudes that differ in the stage's qubits
-// (qubit 0, the pack bit, and two to four register qubits) into registers as packed pairs,
+// (qubit 0, the pack bit, and two or four register qubits) into registers as packed pairs,
 // applies the stage's gates there (the pair update of §2 with packed fp32x2 arithmetic;
 // diagonal gates as signs, phases and projector factors, conditioned on the thread's other
 // index bits), and writes them back (tile_interp.cuh).  Tile size and register width by
@@ -72,7 +72,6 @@ cudaError_t launch_tile_pass(float2 *psi, int n, const unsigned char *block, uin
   if (m < rk + 2 || m > kMaxBits || m > n) return cudaErrorInvalidValue;
   switch (rk) {
     case 2: return launch<2>(psi, n, block, bytes, m, st);
-    case 3: return launch<3>(psi, n, block, bytes, m, st);
     case 4: return launch<4>(psi, n, block, bytes, m, st);
     default: return cudaErrorInvalidValue;
   }

@@ -21,7 +21,7 @@ cudaError_t launch_init(float2 *psi, int n, bool uniform, float amp, cudaStream_
 
 // K1/K2/K3 plain tile pass, interpreted: one sweep over all tiles (m qubits) of one pass;
 // block: the pass's program in device memory (interp_dev.h), of `bytes` bytes; rk: the
-// plan's register slots (2..4).
+// plan's register slots (2 or 4).
 cudaError_t launch_tile_pass(float2 *psi, int n, const unsigned char *block, uint32_t bytes, int m, int rk,
                              cudaStream_t st);
 // Largest tile (qubits) of the interpreting plain kernel; the plan-specialised kernels
