@@ -461,7 +461,8 @@ __device__ __forceinline__ void load_group_rx(const float4 *tile, uint32_t a0, c
     float4 x;
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
                  : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w)
-                 : "r"(pair_address(tb, a0, rx, p)));
+                 : "r"(pair_address(tb, a0, rx, p))
+                 : "memory");
     R[p] = kCopied ? f2(x.x, x.z) : f2(x.x, x.y);
     I[p] = kCopied ? f2(x.y, x.w) : f2(x.z, x.w);
   }
