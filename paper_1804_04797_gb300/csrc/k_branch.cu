@@ -90,7 +90,9 @@ __global__ void __launch_bounds__(256, 2) outer_sum_kernel(const float2 *__restr
                                                            float2 *__restrict__ out) {
   __shared__ float4 As[2][kStep][kColsA / 2], Bs[2][kStep][kRowsB];
   __shared__ uint64_t col_at[kColsA], row_at[kRowsB];  // x_A of the tile's columns, x_B of its rows
-  const uint32_t branches = 1u << S.t;
+  // 2^t branches (t up to 33: their number takes 34 bits) in steps of kStep or fewer
+  const uint32_t steps = 1u << max(S.t - 3, 0), last = steps - 1;
+  const int per_step = 1 << min(S.t, 3);
   const int nA = S.nA, nB = S.nB, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31;
   const uint32_t ct = blockIdx.x & ((1u << tiles_a_log2) - 1), rt = blockIdx.x >> tiles_a_log2;
   // the index bits in the order of S.a_bit and S.b_bit, a slice's (the last ones) above the tiles
@@ -119,22 +121,22 @@ __global__ void __launch_bounds__(256, 2) outer_sum_kernel(const float2 *__restr
   const float2 *pa = A + off_a + col_at[ca] + ((uint64_t)ka << nA), *pb = B + off_b + row_at[rb] + ((uint64_t)kb << nB);
   const uint64_t step_a = 2ull << nA, step_b = 4ull << nB;
   float2 va[kStep / 2], vb[kStep / 4];
-  auto fetch = [&](uint32_t l0) {
+  auto fetch = [&]() {
 #pragma unroll
     for (int k = 0; k < kStep / 2; ++k, pa += step_a)
-      va[k] = in_a && l0 + 2 * k + ka < branches ? *pa : make_float2(0.f, 0.f);
+      va[k] = in_a && 2 * k + ka < per_step ? *pa : make_float2(0.f, 0.f);
 #pragma unroll
     for (int k = 0; k < kStep / 4; ++k, pb += step_b)
-      vb[k] = in_b && l0 + 4 * k + kb < branches ? *pb : make_float2(0.f, 0.f);
+      vb[k] = in_b && 4 * k + kb < per_step ? *pb : make_float2(0.f, 0.f);
   };
   float2 re[4][4], im[4][4];  // [row][pair]
 #pragma unroll
   for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int j = 0; j < 4; ++j) re[r][j] = im[r][j] = make_float2(0.f, 0.f);
-  fetch(0);
+  fetch();
   int s = 0;
-  for (uint32_t l0 = 0; l0 < branches; l0 += kStep, s ^= 1) {
+  for (uint32_t step = 0; step <= last; ++step, s ^= 1) {
 #pragma unroll
     for (int k = 0; k < kStep / 2; ++k) {
       float *const p = reinterpret_cast<float *>(&As[s][2 * k + ka][ca >> 1]) + (ca & 1);
@@ -144,10 +146,9 @@ __global__ void __launch_bounds__(256, 2) outer_sum_kernel(const float2 *__restr
 #pragma unroll
     for (int k = 0; k < kStep / 4; ++k) Bs[s][4 * k + kb][rb] = make_float4(vb[k].x, vb[k].x, vb[k].y, vb[k].y);
     __syncthreads();  // (two buffers: the step before the last has been read by every thread)
-    if (l0 + kStep < branches) fetch(l0 + kStep);
-    const int steps = (int)min((uint32_t)kStep, branches - l0);
+    if (step < last) fetch();
 #pragma unroll 1  // (unrolled 2, 4, 8 times: 1.10, 1.14, 1.23 ms against 1.08 at 28 qubits, 2^4 branches)
-    for (int k = 0; k < steps; ++k) {
+    for (int k = 0; k < per_step; ++k) {
       float4 a[4], b[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) a[j] = As[s][k][16 * j + tx];
