@@ -16,6 +16,11 @@
 
 namespace svp {
 
+#ifdef SV_PLAN_CHECK
+// Greedy choices compared with a search that tries one candidate at a time, and those that differ.
+int plan_checks = 0, plan_check_differences = 0;
+#endif
+
 void kind_matrix(int kind, double m[8]) {
   const double r = 1.0 / std::sqrt(2.0);
   const double c8 = std::cos(M_PI / 4), s8 = std::sin(M_PI / 4);
@@ -491,6 +496,26 @@ bool build_plan(int n, const std::vector<Gate> &gates, const Options &opt, bool 
       }
       return {nd, tot};
     };
+#ifdef SV_PLAN_CHECK
+    auto register_set_one_by_one = [&](const std::vector<char> &dn) -> uint32_t {
+      uint32_t Rm = pack ? 1u : 0u;
+      std::vector<char> tmp = dn;
+      std::pair<int, int> cur = run_stage(Rm, tmp, nullptr, nullptr);
+      for (int round = 0; round < r; ++round) {
+        int best = -1;
+        for (int q = 0; q < n; ++q) {
+          const int b = local_of[q];
+          if (b < 0 || ((Rm >> b) & 1u)) continue;
+          tmp = dn;
+          const std::pair<int, int> sc = run_stage(Rm | (1u << b), tmp, nullptr, nullptr);
+          if (sc > cur) { cur = sc; best = b; }
+        }
+        if (best < 0) break;
+        Rm |= 1u << best;
+      }
+      return Rm;
+    };
+#endif
     // A stage's register set by greedy lookahead from schedule dn: add the tile bit that lets
     // the stage place the most non-diagonal gates (then the most gates), up to r bits; ties go
     // to the lower qubit whatever the tile's bit order, so a layout's reordering of the tile
@@ -554,6 +579,10 @@ bool build_plan(int n, const std::vector<Gate> &gates, const Options &opt, bool 
         Rm |= 1u << best;
         cur = bs;
       }
+#ifdef SV_PLAN_CHECK
+      ++plan_checks;
+      plan_check_differences += Rm != register_set_one_by_one(dn);
+#endif
       return Rm;
     };
     // The register qubits of every stage, by the same greedy choice as below on copies of
