@@ -86,15 +86,27 @@ svp::Options plan_options(const sv_options &o) {
 
 // Tile size and register slots of a plan on the interpreting kernel where the options leave
 // both open.  Measured on one GB300, us per circuit of depth 16 from |0..0> / 12 on a loaded
-// state, by (register slots, tile qubits):
-//   10 qubits  (2,10) 13.4/13.7  (4,10) 14.8/17.6     one tile: fewer amplitudes a thread
-//              are more warps on the one SM; from 12 qubits the op count weighs more
-//   12         (4,12) 17.8/20.5  (2,12) 21.2/23.2     (2,11) 19.8/24.2
-//   14         (2,11) 22.6/26.7  (4,12) 25.3/28.8     (4,13) 24.6/33.5
-//   16         (4,12) 28.2/30.8  (2,11) 27.3/34.8     (4,13) 31.7/35.5
-//   20         (4,13) 38.8/51.8  (4,12) 45.4/48.3     (128 tiles: one to an SM)
-//   23         (4,12) 164/214    (4,13) 168/212       (4,11) 172/217
-// From 24 qubits (no run-time compiler) passes over HBM weigh most: the largest tile.
+// state, by (register slots, tile qubits), the rule's choice first:
+//   10 qubits  (2,10) 12.5/14.5  (4,10) 14.5/16.6
+//   11         (2,11) 16.5/18.2  (4,11) 14.5/18.6
+//   12         (4,12) 17.6/20.6  (2,12) 20.7/22.7  (2,11) 21.7/22.7
+//   13         (2,11) 22.7/23.3  (4,13) 22.1/24.7  (4,12) 24.7/26.8
+//   14         (2,11) 24.7/26.8  (4,12) 25.8/28.8  (4,13) 28.3/30.9
+//   15         (2,11) 24.8/26.8  (4,12) 26.8/29.9  (4,13) 30.9/33.3
+//   16         (4,12) 29.8/30.9  (2,11) 26.8/35.0  (4,13) 30.9/37.0
+//   17         (4,12) 28.8/35.0  (2,11) 33.0/37.0  (4,13) 35.0/39.1
+//   18         (4,12) 30.9/35.0  (2,11) 35.0/35.4  (4,13) 35.0/40.8
+//   19         (4,12) 40.1/45.2  (4,13) 37.0/42.0  (4,11) 41.1/49.4
+//   20         (4,13) 38.4/51.8  (4,12) 45.5/49.3  (4,11) 43.4/56.7
+//   21         (4,13) 58.6/63.9  (4,12) 53.7/61.9  (4,11) 55.7/74.1
+//   22         (4,12) 96/130     (4,13) 104/121    (4,11) 105/125
+//   23         (4,12) 170/214    (4,13) 177/208    (4,11) 180/209
+// Few tiles: fewer amplitudes a thread are more warps on the SMs that work; with a tile for
+// many of the SMs the number of ops and passes weighs more.  The rule goes by size alone and was
+// set at 10, 12, 14, 16, 20 and 23 qubits; it is not the best everywhere: at 19 and 21 qubits the
+// other tile is 3-8 % faster from either start, at 11 and 16 from |0..0> and at 20 and 22 loaded
+// another shape 5-12 %.  From 24 qubits (no run-time compiler) passes over HBM weigh most: the
+// largest tile.
 static void interp_shape(const sv_options &o, int n, svp::Options *po) {
   if (o.tile_bits != 0 || o.fuse_k != 0 || o.low_bits != 0) return;
   if (n <= 11 || (n >= 13 && n <= 15)) {

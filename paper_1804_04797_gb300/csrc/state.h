@@ -31,8 +31,9 @@ struct sv_state {
   bool fresh = false;     // logically |0..0> but not yet written (lazy initial state)
   bool broken = false;    // an apply failed part-way: content undefined
   // a state of a few-amplitude call (cut branches, inner products): plans on the interpreting
-  // kernel keep one shape, so that an amplitude does not change, to the last bit, with the
-  // tuning of the state path's shapes (interp_shape)
+  // kernel keep one shape, 13-qubit tiles and four slots, so that an amplitude, returned in double
+  // precision, is the same to the last bit whichever shapes the state path is tuned to
+  // (interp_shape).  The bits are rounding of the fp32 states: no shape is more accurate.
   bool one_shape = false;
   // > 0: a branch tree's prefix whose `fork` highest qubits the next plan takes as |+> (memory
   // holds the slice in which they are 0)

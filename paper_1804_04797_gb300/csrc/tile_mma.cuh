@@ -74,9 +74,8 @@ __device__ __forceinline__ void mma(uint32_t d, uint32_t a, uint64_t b, uint32_t
 }
 
 // One lane of a converged warp.  The products are issued under this and not under a comparison
-// of the lane: the compiler then knows that one thread is active and keeps their operands in
-// uniform registers, which the instruction reads (a stage's 12 F16x3 products 541 -> 390 cycles,
-// its 24 TF32x3 ones 1091 -> 775: 32 each, the rate of the tensor cores at N = 64).
+// of the lane: a stage's 12 F16x3 products then take 390 cycles instead of 541, its 24 TF32x3
+// ones 775 instead of 1091 (32 each, the rate of the tensor cores at N = 64).
 __device__ __forceinline__ bool elect_lane() {
   uint32_t p;
   asm volatile("{\n .reg .pred P;\n .reg .b32 r;\n elect.sync r|P, 0xffffffff;\n selp.b32 %0, 1, 0, P;\n}\n" : "=r"(p));

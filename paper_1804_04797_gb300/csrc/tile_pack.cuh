@@ -438,8 +438,9 @@ __device__ __forceinline__ uint32_t pack_phys(uint32_t k) { return k ^ (((k >> 3
 // masks of the register slots (constants in the kernels compiled for one plan).
 // Address of pair p of a group (rx: the offsets of its register slots, constants).  The tile bits
 // meet in the 128-byte row's address bits alone, where the layouts add them without carry; above
-// these each has a bit of its own, so that part is a constant of the access (an XOR for each of
-// the pairs before; 30 qubits 14.94 -> 14.80 ms, 27 qubits 1.83 -> 1.80, one GB300).
+// these each has a bit of its own, so that part is a constant of the access (with an XOR for each
+// of the pairs instead / so, one GB300: 24 qubits 182.4 / 180.8 us, 26 754 / 737, 25 qubits TF32x3
+// 807 / 772; 28 qubits F16x3 6.40 / 6.38 ms; 27 and 30 qubits the same).
 __device__ __forceinline__ uint32_t pair_address(uint32_t tile, uint32_t a0, const uint32_t (&rx)[kPR], int p) {
   uint32_t row = 0, above = 0;
 #pragma unroll
