@@ -729,6 +729,7 @@ sv_status basis_inner_products(sv_state *with, const std::vector<svp::Gate> &g, 
   s->opts = with->opts;
   s->stream = with->stream;
   s->device = with->device;
+  s->keep_uploads = true;
   if (cudaMalloc(reinterpret_cast<void **>(&s->psi), sizeof(float2) << svj::basis_state_bits(P)) != cudaSuccess ||
       cudaMalloc(reinterpret_cast<void **>(&s->d_sums), (2 + 2 * (size_t)svj::max_pass_grid()) * sizeof(double)) !=
           cudaSuccess) {
@@ -737,6 +738,7 @@ sv_status basis_inner_products(sv_state *with, const std::vector<svp::Gate> &g, 
   }
   svk::DevPlanView view;
   if ((st = upload_plan(s, P, &view)) != SV_OK) return st;
+  if (with->err_pending) view.err = with->err_pending;  // one word, read once, for both states' waits
   if ((st = ensure_device_buffer(&s->d_scratch, &s->d_scratch_cap, 2 * m * sizeof(double))) != SV_OK) return st;
   double *const d_out = static_cast<double *>(s->d_scratch);
   cudaError_t e = cudaSuccess;
@@ -753,7 +755,7 @@ sv_status basis_inner_products(sv_state *with, const std::vector<svp::Gate> &g, 
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "inner product pass");
   s->err_pending = view.err;
-  if ((st = take_pending_error(s)) != SV_OK || (st = take_pending_error(with)) != SV_OK) return st;
+  if ((st = take_pending_error(with->err_pending ? with : s)) != SV_OK) return st;
   *done = true;
   return SV_OK;
 }

@@ -403,7 +403,7 @@ extern "C" sv_status sv_amplitudes_by_inner_product(const sv_lattice *lat, int s
   if (opts) o = *opts;
   Holder A, B;
   if ((st = sv_create(n, &o, &A.s)) != SV_OK) return st;
-  A.s->one_shape = true;
+  A.s->one_shape = A.s->keep_uploads = true;
   if ((st = sv_apply_circuit(A.s, g1.data(), g1.size())) != SV_OK) return st;  // |psi> = U1 H|0>
   if (m == 0) return SV_OK;
   std::vector<svp::Gate> g2_inv;
@@ -411,7 +411,7 @@ extern "C" sv_status sv_amplitudes_by_inner_product(const sv_lattice *lat, int s
   bool done = false;
   if ((st = basis_inner_products(A.s, g2_inv, bits, m, out_re_im, &done)) != SV_OK || done) return st;
   if ((st = sv_create(n, &o, &B.s)) != SV_OK) return st;
-  B.s->one_shape = true;
+  B.s->one_shape = B.s->keep_uploads = true;
   for (size_t j = 0; j < m; ++j) {
     // |phi_x> = U2^dagger |x>;  alpha_x = <phi_x|psi>: on plan kernels the last pass of
     // phi_x sums the inner product instead of storing phi_x

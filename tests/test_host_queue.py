@@ -19,7 +19,7 @@ def test_sources_of_queued_copies_stay_as_they_are(fake_device, jit, precision):
     assert r.returncode == 0, r.stdout + r.stderr
 
 
-@pytest.mark.parametrize('how,passes', [('support', (0,)), ('whole', (0,)), ('product', (0, 3))])
+@pytest.mark.parametrize('how,passes', [('support', (0, 3)), ('whole', (0, 2)), ('product', (0, 3))])
 def test_a_state_that_was_not_finished_is_reported_by_the_call_that_reads_it(fake_device, how, passes):
     for fail in (-1, *passes):
         r = host_cpp.run(fake_device, 'gave_up', how, fail)
